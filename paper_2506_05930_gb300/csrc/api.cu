@@ -522,12 +522,8 @@ nvc_status nvc_infer(nvc_handle* h, const float* pos, int64_t n, float* vis, voi
     count_launches(h, 1);
     return NVC_OK;
   }
-  for (int64_t o = 0; o < n; o += h->stage_pixels) {
-    const int64_t m = n - o < h->stage_pixels ? n - o : h->stage_pixels;
-    NVC_CUDA(h, launch_encode_fwd(h, pos + 3 * o, m, h->s_feat, s));
-    NVC_CUDA(h, launch_mlp_fwd_fp32(h, h->s_feat, m, vis + o * h->L, true, nullptr, s));
-    count_launches(h, 2);
-  }
+  NVC_CUDA(h, launch_infer_f32(h, pos, n, vis, s));
+  count_launches(h, 1);
   return NVC_OK;
 }
 
@@ -591,16 +587,9 @@ static nvc_status shade_impl(nvc_handle* h, const nvc_scene* scene, const float*
     return NVC_OK;
   }
   StageScope sc(h, s, 3);
-  for (int64_t o = 0; o < n; o += h->stage_pixels) {
-    const int64_t m = n - o < h->stage_pixels ? n - o : h->stage_pixels;
-    NVC_CUDA(h, launch_encode_fwd(h, pos + 3 * o, m, h->s_feat, s));
-    NVC_CUDA(h, launch_mlp_fwd_fp32(h, h->s_feat, m, h->s_vis, true, nullptr, s));
-    NVC_CUDA(h, launch_shade_from_vis(scene, pos + 3 * o, nrm + 3 * o, h->s_vis, m, seed, frame,
-                                      view, pixel_offset + o, idx ? idx + o : nullptr,
-                                      pdf ? pdf + o : nullptr, wsum ? wsum + o : nullptr,
-                                      radiance ? radiance + o : nullptr, s));
-    count_launches(h, 3);
-  }
+  NVC_CUDA(h, launch_shade_f32(h, scene, pos, nrm, n, seed, frame, view, pixel_offset, idx, pdf,
+                               wsum, radiance, s));
+  count_launches(h, 1);
   return NVC_OK;
 }
 

@@ -308,10 +308,15 @@ cudaError_t launch_light_weights(const nvc_scene* sc, const float* pos, const fl
 cudaError_t launch_wrs_from_weights(const float* w, int64_t n, int L, uint64_t seed,
                                     uint32_t frame, uint32_t view, int64_t pixel_offset,
                                     int32_t* idx, float* pdf, float* wsum, cudaStream_t s);
-cudaError_t launch_shade_from_vis(const nvc_scene* sc, const float* pos, const float* nrm,
-                                  const float* vis, int64_t n, uint64_t seed, uint32_t frame,
-                                  uint32_t view, int64_t pixel_offset, int32_t* idx,
-                                  float* pdf, float* wsum, float* radiance, cudaStream_t s);
+
+// fp32_shade.cu: float32 inference, and inference + sampling + Neural DI, in
+// one kernel each.
+cudaError_t launch_infer_f32(const nvc_handle* h, const float* pos, int64_t n, float* vis,
+                             cudaStream_t s);
+cudaError_t launch_shade_f32(const nvc_handle* h, const nvc_scene* sc, const float* pos,
+                             const float* nrm, int64_t n, uint64_t seed, uint32_t frame,
+                             uint32_t view, int64_t pixel_offset, int32_t* idx, float* pdf,
+                             float* wsum, float* radiance, cudaStream_t s);
 
 // train.cu
 // n_world: world-space positions in the batch, -1 for ceil(batch / 2); every
