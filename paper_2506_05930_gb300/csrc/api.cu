@@ -1074,6 +1074,13 @@ static nvc_status train_forward_backward(nvc_handle* h, const nvc_scene* scene,
     count_launches(h, 1);
     return NVC_OK;
   }
+  if (train_f32_fits(h)) {
+    int blocks = 0;
+    NVC_CUDA(h, launch_train_f32(h, B, &blocks, s));
+    h->loss_blocks = blocks;
+    count_launches(h, 1);
+    return NVC_OK;
+  }
   NVC_CUDA(h, launch_encode_fwd(h, h->t_pos, B, h->t_feat, s));
   NVC_CUDA(h, launch_mlp_fwd_fp32(h, h->t_feat, B, h->t_logits, false, h->t_act, s));
   NVC_CUDA(h, launch_loss_grad(h, B, s));

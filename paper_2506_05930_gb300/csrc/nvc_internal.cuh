@@ -318,6 +318,11 @@ cudaError_t launch_shade_f32(const nvc_handle* h, const nvc_scene* sc, const flo
                              uint32_t view, int64_t pixel_offset, int32_t* idx, float* pdf,
                              float* wsum, float* radiance, cudaStream_t s);
 
+// fp32_train.cu: one float32 training pass (encode, forward, loss, backward,
+// scatter) in one kernel; false when the network does not fit on chip.
+bool train_f32_fits(const nvc_handle* h);
+cudaError_t launch_train_f32(nvc_handle* h, int64_t n, int* blocks_used, cudaStream_t s);
+
 // train.cu
 // n_world: world-space positions in the batch, -1 for ceil(batch / 2); every
 // position is world-space when no screen positions are given.

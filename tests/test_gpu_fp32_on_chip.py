@@ -62,3 +62,36 @@ def test_inference_and_shading_equal_the_separate_kernels(F, levels, hidden, L, 
     di = (ref.double() * c.double()).sum(1)
     assert torch.all((out["radiance"].double() - di).abs() <= (L + 1) * 2.0 ** -23 * di + 1e-30)
     cache.close()
+
+
+@pytest.mark.parametrize("F,levels,hidden,L", SHAPES)
+@pytest.mark.parametrize("loss", ["l2", "bce"])
+@pytest.mark.parametrize("batch", [1, 33, 9000])
+def test_training_gradient_equals_the_separate_kernels(F, levels, hidden, L, loss, batch):
+    """Against nvc_mlp_forward / nvc_mlp_backward on the same batch with the
+    loss gradient formed in float64.  Both sides round every product and add
+    the same terms in another order: 1e-5 of the gradient's norm, as the
+    oracle comparisons allow."""
+    from paper_2506_05930_gb300 import nvc
+    if L > 128:
+        pytest.skip("this network does not fit on chip: the separate kernels run on both sides")
+    cache, p = _cache(F, levels, hidden, L, seed=batch, loss=loss, batch_positions=batch,
+                      loss_scale=16.0)
+    scene = _scene(L, seed=L + 1)
+    grad, loss_out = cache.train_gradient(scene, None, seed=5, frame=3)
+    pos = torch.empty((batch, 3), device="cuda")
+    y = torch.empty((batch, L), device="cuda")
+    nvc.nvc_training_batch(cache.handle, pos, y)
+    z = torch.empty((batch, L), device="cuda")
+    nvc.nvc_mlp_forward(cache.handle, pos, z)
+    z64, y64 = z.double().requires_grad_(True), y.double()
+    ref_loss = (torch.nn.functional.binary_cross_entropy_with_logits(z64, y64) if loss == "bce"
+                else ((torch.sigmoid(z64) - y64) ** 2).mean())
+    dz, = torch.autograd.grad(ref_loss, z64)
+    ref = torch.empty(cache.n_params, device="cuda")
+    nvc.nvc_mlp_backward(cache.handle, pos, dz.float().contiguous(), ref)
+    assert abs(loss_out.item() - ref_loss.item()) <= 1e-6 * abs(ref_loss.item())
+    err = (grad.double() - ref.double()).norm().item()
+    assert err <= 1e-5 * ref.double().norm().item()
+    assert cache.counters()["error_flags"] == 0
+    cache.close()
