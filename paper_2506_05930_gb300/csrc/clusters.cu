@@ -9,18 +9,22 @@
 //   cluster_targets_kernel   training targets: for each (position, cluster)
 //                            the binary visibility of one member drawn
 //                            uniformly, so the network learns the average;
-//   sample_clustered_kernel  per pixel: c_hat_y = sum of the members'
+//   sample_sum_kernel        per pixel: c_hat_y = sum of the members'
 //                            contributions, w_y = max(v_y, 0.001) c_hat_y,
 //                            the integer reservoir over the clusters, then
 //                            kRis uniform members of cluster y, one kept by
 //                            the integer reservoir on their contributions,
 //                            and its unbiased contribution weight
 //                            W = (sum_j c_j / M) / (p(x) c(x)),
-//                            p(x) = (w(y) / w_sum) / m_y.
+//                            p(x) = (w(y) / w_sum) / m_y;
+//   sample_visibility_kernel the same with w_y = max(v_y, 0.001) alone.
 // Every float32 result is rounded in a fixed order and every random choice
-// is a fixed Philox word, so both kernels are reproducible bit for bit.
+// is a fixed Philox word, so the kernels are reproducible bit for bit.
+#include <cfloat>
 #include <vector>
 
+#include "exact_pair.cuh"
+#include "fused_common.cuh"
 #include "nvc_internal.cuh"
 #include "shadow.cuh"
 
@@ -95,27 +99,22 @@ __device__ __forceinline__ int integer_reservoir(const float (&w)[N], int n, con
   return sel;
 }
 
-// Light e with I / pi in .w: from the shared copy, or from global memory
-// (scaled here, the same rounding) when the lights do not fit on chip.
-template <bool kSmemLights>
-__device__ __forceinline__ float4 light_at(const float4* s_lt, const float* lights, int e) {
-  if (kSmemLights) return s_lt[e];
-  float4 l = __ldg(reinterpret_cast<const float4*>(lights) + e);
-  l.w = __fmul_rn(l.w, bits_f(kInvPiBits));
-  return l;
-}
-
-// Integer reservoir over the k cluster weights w with the words of stream
-// (pixel, frame, view, kTagWrs), drawn four at a time as the scan reaches
-// them: the same picks as integer_reservoir with r[y] = word y.
-__device__ __forceinline__ int cluster_reservoir(const float (&w)[kMaxClusters], int k,
-                                                 uint32_t pixel, uint32_t frame, uint32_t view,
-                                                 uint32_t k0, uint32_t k1) {
+// Integer reservoir over the k cluster weights wfn(y) with the words of
+// stream (pixel, frame, view, kTagWrs), drawn four at a time as the scan
+// reaches them: the same picks as integer_reservoir with r[y] = word y.  wfn
+// is called with constants below kMaxClusters (weights may be registers).
+template <typename WFn>
+__device__ __forceinline__ int cluster_reservoir(WFn wfn, int k, uint32_t pixel, uint32_t frame,
+                                                 uint32_t view, uint32_t k0, uint32_t k1) {
   float wmax = 0.0f;
 #pragma unroll
   for (int y = 0; y < kMaxClusters; ++y)
-    if (y < k) wmax = fmaxf(wmax, w[y]);
+    if (y < k) wmax = fmaxf(wmax, wfn(y));
   if (!(wmax > 0.0f)) return -1;
+  // quantize_weight's integers by exact multiplications; an infinite weight
+  // takes quantize_weight itself
+  const bool finite = wmax <= FLT_MAX;
+  const fz::QuantScale qs = fz::quant_scale(wmax);
   const int e = ilogbf(wmax);
   uint32_t Q = 0;
   int sel = -1;
@@ -123,14 +122,15 @@ __device__ __forceinline__ int cluster_reservoir(const float (&w)[kMaxClusters],
   for (int g = 0; g < kMaxClusters / 4; ++g) {
     if (4 * g < k) {
       const uint4 r4 = philox4x32_10(make_uint4(pixel, frame, view, ((uint32_t)g << 4) | kTagWrs), k0, k1);
-      const uint32_t r[4] = {r4.x, r4.y, r4.z, r4.w};
 #pragma unroll
       for (int l = 0; l < 4; ++l) {
         const int y = 4 * g + l;
         if (y < k) {
-          const uint32_t q = quantize_weight(w[y], e);
+          const float w = wfn(y);
+          const uint32_t q = finite ? fz::quantize_scaled(__fmul_rn(w, qs.pre), qs.scale)
+                                    : quantize_weight(w, e);
           Q += q;
-          if (q > 0u && __umulhi(r[l], Q) < q) sel = y;
+          if (q > 0u && __umulhi(fz::pick_word(r4, l), Q) < q) sel = y;
         }
       }
     }
@@ -138,199 +138,278 @@ __device__ __forceinline__ int cluster_reservoir(const float (&w)[kMaxClusters],
   return sel;
 }
 
-// Lights per shared-memory tile of the tiled step 1 (16 KB).
-constexpr int kLightTile = 1024;
+// What both first steps share: the scene, the cluster table and the outputs.
+struct ClusterArgs {
+  const float* lights;
+  int n_lights;
+  const float* spheres;
+  int n_sph;
+  const float* boxes;
+  int n_box;
+  const int32_t* off;
+  const int32_t* mem;
+  int k;
+  const float* vis;
+  const float* pos;
+  const float* nrm;
+  int64_t n;
+  int64_t pixel_offset;
+  uint32_t k0, k1, frame, view;
+  int32_t* light_out;
+  float* weight_out;
+  float* estimate;
+  float neg0;               // -0.0f (exact_pair.cuh)
+  int tile;                 // staged light slots (sum weights)
+};
 
-// Shared-memory layout: [the lights in cluster-table order, I / pi in .w
-// (kSmemLights: all of them; kTiled: one tile of kLightTile)] [spheres]
-// [offsets k + 1, as float4 slots] [boxes].  With the lights in table order
-// the members of cluster y are the contiguous slots offsets[y] ..
-// offsets[y + 1] - 1.
-// kSum: first-step weights max(v, 0.001) * c_hat (else max(v, 0.001) alone,
-// and no light loop).
-// kTiled (with kSum, for light sets too large to stage whole): the CTA's
-// threads walk the table in tiles of kLightTile lights staged together in
-// shared memory, each thread carrying its pixel's running cluster sum across
-// tiles -- the same additions in the same order as the whole-set loop.
-template <bool kSmemLights, bool kSum, bool kTiled = false>
-__global__ void __launch_bounds__(1024) sample_clustered_kernel(
-    const float* __restrict__ lights, int n_lights, const float* __restrict__ spheres, int n_sph,
-    const float* __restrict__ boxes, int n_box, const int32_t* __restrict__ off,
-    const int32_t* __restrict__ mem, int k, const float* __restrict__ vis,
-    const float* __restrict__ pos, const float* __restrict__ nrm, int64_t n,
-    int64_t pixel_offset, uint32_t k0, uint32_t k1, uint32_t frame, uint32_t view,
-    int32_t* __restrict__ light_out, float* __restrict__ weight_out, float* __restrict__ estimate,
-    bool vis_vec4) {
-  extern __shared__ float4 s_scene4[];
-  const int n_lt_s = kSmemLights ? n_lights : kTiled ? kLightTile : 0;
-  float4* s_lt = s_scene4;
-  int32_t* s_off = reinterpret_cast<int32_t*>(s_lt + n_lt_s);
-  const Occluders occ = stage_occluders(spheres, n_sph, boxes, n_box,
-                                        s_lt + n_lt_s + (kMaxClusters + 4) / 4, threadIdx.x,
-                                        blockDim.x);
-  if (kSmemLights) {
-    for (int e = threadIdx.x; e < n_lt_s; e += blockDim.x) {
-      float4 l = reinterpret_cast<const float4*>(lights)[mem[e]];
-      l.w = __fmul_rn(l.w, bits_f(kInvPiBits));
-      s_lt[e] = l;
+// Step 2 and the outputs of pixel p: streaming RIS among kRis uniform members
+// of cluster y (y < 0: nothing contributes) with weight w_y of wsum, the
+// unbiased contribution weight, and the one-ray estimate.  light(slot): the
+// light at a place of the cluster table, I / pi in w.
+template <typename LightFn>
+__device__ __forceinline__ void finish_pixel(const ClusterArgs& a, int64_t p, int y, float w_y,
+                                             float wsum, int base, uint32_t m_y, float px, float py,
+                                             float pz, xp::Pixel pp, LightFn light,
+                                             const Occluders& occ) {
+  const uint32_t pixel = (uint32_t)(a.pixel_offset + p);
+  int sel_light = -1;
+  float W = 0.0f, cx = 0.0f;
+  if (y >= 0) {
+    const uint4 u = philox4x32_10(make_uint4(pixel, a.frame, a.view, (0u << 4) | kTagRis), a.k0, a.k1);
+    const uint4 v = philox4x32_10(make_uint4(pixel, a.frame, a.view, (1u << 4) | kTagRis), a.k0, a.k1);
+    const uint32_t ru[kRis] = {u.x, u.y, u.z, u.w};
+    const uint32_t rr[kRis] = {v.x, v.y, v.z, v.w};
+    int slot[kRis];
+    float4 lt[kRis];
+#pragma unroll
+    for (int t = 0; t < kRis; ++t) {
+      slot[t] = base + (int)(((uint64_t)ru[t] * m_y) >> 32);
+      lt[t] = light(slot[t]);
+      pp.ok = pp.ok && xp::light_ok(lt[t]);
+    }
+    const float4 ab[kRis] = {make_float4(lt[0].x, lt[1].x, lt[0].y, lt[1].y),
+                             make_float4(lt[0].z, lt[1].z, lt[0].w, lt[1].w),
+                             make_float4(lt[2].x, lt[3].x, lt[2].y, lt[3].y),
+                             make_float4(lt[2].z, lt[3].z, lt[2].w, lt[3].w)};
+    float cc[kRis];
+    xp::contributions<kRis / 2>(pp, ab, cc);
+    const int j = integer_reservoir(cc, kRis, rr);
+    if (j >= 0) {
+      float sum = 0.0f;
+#pragma unroll
+      for (int t = 0; t < kRis; ++t) sum = __fadd_rn(sum, cc[t]);
+      float c_j = 0.0f;
+      int s_j = 0;
+#pragma unroll
+      for (int t = 0; t < kRis; ++t)
+        if (t == j) {
+          c_j = cc[t];
+          s_j = slot[t];
+        }
+      const float mean = __fdiv_rn(sum, (float)kRis);
+      const float pr = __fdiv_rn(__fdiv_rn(w_y, wsum), (float)m_y);
+      W = __fdiv_rn(mean, __fmul_rn(pr, c_j));
+      sel_light = a.mem[s_j];
+      cx = c_j;
     }
   }
-  for (int e = threadIdx.x; e <= k; e += blockDim.x) s_off[e] = off[e];
+  if (a.light_out) a.light_out[p] = sel_light;
+  if (a.weight_out) a.weight_out[p] = W;
+  if (a.estimate) {
+    float e = 0.0f;
+    if (sel_light >= 0) {
+      const float4 l = reinterpret_cast<const float4*>(a.lights)[sel_light];
+      if (!segment_blocked(px, py, pz, l.x, l.y, l.z, occ)) e = __fmul_rn(cx, W);
+    }
+    a.estimate[p] = e;
+  }
+}
+
+// A light of the cluster table from global memory, I / pi in w.
+__device__ __forceinline__ float4 table_light(const ClusterArgs& a, int slot) {
+  float4 l = __ldg(reinterpret_cast<const float4*>(a.lights) + a.mem[slot]);
+  l.w = __fmul_rn(l.w, bits_f(kInvPiBits));
+  return l;
+}
+
+// ---- first-step weights max(v, 0.001) alone ---------------------------------
+// No light loop: a pixel's visibilities are loaded together (16-byte loads
+// when the row allows) into the weights' registers.
+__global__ void __launch_bounds__(128, 7) sample_visibility_kernel(const __grid_constant__ ClusterArgs a,
+                                                                 bool vis_vec4) {
+  extern __shared__ float4 s_scene4[];
+  int32_t* s_off = reinterpret_cast<int32_t*>(s_scene4);
+  const Occluders occ = stage_occluders(a.spheres, a.n_sph, a.boxes, a.n_box,
+                                        s_scene4 + (kMaxClusters + 4) / 4, threadIdx.x, blockDim.x);
+  const int k = a.k;
+  for (int e = threadIdx.x; e <= k; e += blockDim.x) s_off[e] = a.off[e];
   __syncthreads();
-  // the CTA walks its pixel batches together (the tiled step 1 has block
-  // barriers); a thread past the end takes part in them and writes nothing
-  for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < n;
-       base += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t p = base + threadIdx.x;
-    const bool live = p < n;
-    if (!kTiled && !live) continue;
-    const int64_t pl = live ? p : 0;
-    const float px = pos[3 * pl], py = pos[3 * pl + 1], pz = pos[3 * pl + 2];
-    const float nx = nrm[3 * pl], ny = nrm[3 * pl + 1], nz = nrm[3 * pl + 2];
-    const uint32_t pixel = (uint32_t)(pixel_offset + p);
-    // step 1: the clusters' weights, then the reservoir over them.  The
-    // cluster loop stays a loop (one copy of the member loop in the code, so
-    // warps at different clusters share the instruction cache); the weights
-    // stay in registers through compare-and-select writes.
+  for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < a.n;
+       p += (int64_t)gridDim.x * blockDim.x) {
+    const float px = a.pos[3 * p], py = a.pos[3 * p + 1], pz = a.pos[3 * p + 2];
+    const float nx = a.nrm[3 * p], ny = a.nrm[3 * p + 1], nz = a.nrm[3 * p + 2];
     float w[kMaxClusters];
     float wsum = 0.0f;
-    const float* vrow = vis + pl * k;
-    if (kTiled) {
+    const float* vrow = a.vis + p * k;
+    if (vis_vec4) {
 #pragma unroll
-      for (int t = 0; t < kMaxClusters; ++t) w[t] = 0.0f;
-      int y = 0;
-      float ch = 0.0f;
-      // cluster y is complete: its weight, in cluster order
-      auto finish = [&]() {
-        const float wy = __fmul_rn(fmaxf(__ldg(vrow + y), bits_f(kVisClampBits)), ch);
-#pragma unroll
-        for (int t = 0; t < kMaxClusters; ++t)
-          if (t == y) w[t] = wy;
-        wsum = __fadd_rn(wsum, wy);
-        ch = 0.0f;
-        ++y;
-      };
-      for (int c0 = 0; c0 < n_lights; c0 += kLightTile) {
-        const int cn = n_lights - c0 < kLightTile ? n_lights - c0 : kLightTile;
-        __syncthreads();   // the previous tile is read by every thread
-        for (int e = threadIdx.x; e < cn; e += blockDim.x) {
-          float4 l = __ldg(reinterpret_cast<const float4*>(lights) + mem[c0 + e]);
-          l.w = __fmul_rn(l.w, bits_f(kInvPiBits));
-          s_lt[e] = l;
-        }
-        __syncthreads();
-        if (live) {
-#pragma unroll 4
-          for (int i = 0; i < cn; ++i) {
-            while (c0 + i >= s_off[y + 1]) finish();
-            const float4 l = s_lt[i];
-            ch = __fadd_rn(ch, contribution(px, py, pz, nx, ny, nz, l.x, l.y, l.z, l.w));
-          }
-        }
-      }
-      if (live)
-        while (y < k) finish();
-    } else if (!kSum) {
-      // visibility weights: no member loop, so the row's loads are issued
-      // together (16-byte loads when the row allows) into the weights'
-      // registers, and the short cluster loop is unrolled
-      if (vis_vec4) {
-#pragma unroll
-        for (int g = 0; g < kMaxClusters / 4; ++g) {
-          float4 v = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-          if (4 * g < k) v = __ldg(reinterpret_cast<const float4*>(vrow) + g);
-          w[4 * g] = v.x;
-          w[4 * g + 1] = v.y;
-          w[4 * g + 2] = v.z;
-          w[4 * g + 3] = v.w;
-        }
-      } else {
-#pragma unroll
-        for (int t = 0; t < kMaxClusters; ++t) w[t] = t < k ? __ldg(vrow + t) : 0.0f;
-      }
-#pragma unroll
-      for (int t = 0; t < kMaxClusters; ++t) {
-        if (t < k) {
-          w[t] = s_off[t + 1] > s_off[t] ? fmaxf(w[t], bits_f(kVisClampBits)) : 0.0f;
-          wsum = __fadd_rn(wsum, w[t]);
-        } else {
-          w[t] = 0.0f;
-        }
+      for (int g = 0; g < kMaxClusters / 4; ++g) {
+        float4 v = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        if (4 * g < k) v = __ldg(reinterpret_cast<const float4*>(vrow) + g);
+        w[4 * g] = v.x;
+        w[4 * g + 1] = v.y;
+        w[4 * g + 2] = v.z;
+        w[4 * g + 3] = v.w;
       }
     } else {
 #pragma unroll
-      for (int t = 0; t < kMaxClusters; ++t) w[t] = 0.0f;
-#pragma unroll 1
-      for (int y = 0; y < k; ++y) {
-        const float v = __ldg(vrow + y);
-        const int begin = s_off[y], end = s_off[y + 1];
-        float ch = 0.0f;
-#pragma unroll 4
-        for (int i = begin; i < end; ++i) {
-          const float4 l = kSmemLights ? s_lt[i] : light_at<false>(s_lt, lights, mem[i]);
-          ch = __fadd_rn(ch, contribution(px, py, pz, nx, ny, nz, l.x, l.y, l.z, l.w));
+      for (int t = 0; t < kMaxClusters; ++t) w[t] = t < k ? __ldg(vrow + t) : 0.0f;
+    }
+#pragma unroll
+    for (int t = 0; t < kMaxClusters; ++t) {
+      if (t < k) {
+        w[t] = s_off[t + 1] > s_off[t] ? fmaxf(w[t], bits_f(kVisClampBits)) : 0.0f;
+        wsum = __fadd_rn(wsum, w[t]);
+      } else {
+        w[t] = 0.0f;
+      }
+    }
+    const int y = cluster_reservoir([&](int t) { return w[t]; }, k, (uint32_t)(a.pixel_offset + p),
+                                    a.frame, a.view, a.k0, a.k1);
+    float w_y = 0.0f;
+#pragma unroll
+    for (int t = 0; t < kMaxClusters; ++t)
+      if (t == y) w_y = w[t];
+    const int base = y < 0 ? 0 : s_off[y];
+    finish_pixel(a, p, y, w_y, wsum, base, y < 0 ? 0u : (uint32_t)(s_off[y + 1] - base), px, py, pz,
+                 xp::make_pixel(px, py, pz, nx, ny, nz, a.neg0, true),
+                 [&](int slot) { return table_light(a, slot); }, occ);
+  }
+}
+
+// ---- first-step weights max(v, 0.001) x sum of the members' contributions ---
+// The cost is one correctly rounded contribution per light and pixel, two
+// lights per packed operation (exact_pair.cuh).  The lights are staged in
+// cluster-table order as pairs, every cluster's run padded to an even count
+// with a zero light (its contribution +0 leaves the sum as it is), so no pair
+// straddles two clusters; more slots than a tile are walked tile by tile,
+// staged together by the CTA, each thread carrying its pixel's running sum
+// across tiles.  All threads of a CTA are at the same cluster and slot.  A
+// pixel's weights lie in shared memory, [cluster][thread].
+//
+// Bound by the FMA pipe and its operand reads: a packed operation takes both
+// halves' cycles (three distinct operands half as many again), 59 a pair by
+// count, some 84 measured.  1920x1080 x 1024 lights, k = 32, with the shadow
+// ray: 3.56 -> 2.54 ms a launch.  Two pairs in flight at 24 warps an SM was
+// the fastest of 1, 2 and 4 pairs at 16, 24 and 32 warps (within 5%).
+constexpr int kLightTile = 1024;
+constexpr int kSumThreads = 256;
+
+// Light slots [t0, t0 + tn) of the padded table into s_lt; whether this
+// thread's lights are inside the packed contribution's bounds.
+__device__ __forceinline__ bool stage_slots(const ClusterArgs& a, const int32_t* s_off,
+                                            const int32_t* s_pad, float4* s_lt, int t0, int tn) {
+  bool ok = true;
+  for (int e = threadIdx.x; e < tn; e += blockDim.x) {
+    int lo = 0, hi = a.k - 1;   // the cluster whose padded run holds slot t0 + e
+    while (lo < hi) {
+      const int mid = (lo + hi + 1) >> 1;
+      if (s_pad[mid] <= t0 + e) lo = mid; else hi = mid - 1;
+    }
+    const int at = s_off[lo] + (t0 + e - s_pad[lo]);
+    const bool pad = at >= s_off[lo + 1];
+    float4 l = table_light(a, pad ? s_off[lo] : at);
+    if (pad) l.w = 0.0f;
+    xp::put_light(s_lt, e, l);
+    ok = ok && xp::light_ok(l);
+  }
+  return ok;
+}
+
+__global__ void __launch_bounds__(kSumThreads, 3)
+    sample_sum_kernel(const __grid_constant__ ClusterArgs a) {
+  extern __shared__ float4 s_scene4[];
+  float4* s_lt = s_scene4;
+  float* s_w = reinterpret_cast<float*>(s_lt + a.tile) + threadIdx.x;
+  int32_t* s_off = reinterpret_cast<int32_t*>(s_lt + a.tile) + kMaxClusters * kSumThreads;
+  int32_t* s_pad = s_off + kMaxClusters + 4;
+  const Occluders occ = stage_occluders(a.spheres, a.n_sph, a.boxes, a.n_box,
+                                        s_pad + kMaxClusters + 4, threadIdx.x, blockDim.x);
+  const int k = a.k;
+  for (int e = threadIdx.x; e <= k; e += blockDim.x) s_off[e] = a.off[e];
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    int at = 0;
+    for (int y = 0; y < k; ++y) {
+      s_pad[y] = at;
+      at += (s_off[y + 1] - s_off[y] + 1) & ~1;
+    }
+    s_pad[k] = at;
+  }
+  __syncthreads();
+  const int n_slots = s_pad[k];
+  const bool whole = n_slots <= a.tile;
+  bool lights_ok = true;
+  if (whole) lights_ok = __syncthreads_and(stage_slots(a, s_off, s_pad, s_lt, 0, n_slots)) != 0;
+  for (int64_t b = (int64_t)blockIdx.x * kSumThreads; b < a.n; b += (int64_t)gridDim.x * kSumThreads) {
+    const int64_t p = b + threadIdx.x;
+    const bool live = p < a.n;
+    const int64_t pl = live ? p : 0;
+    const float px = a.pos[3 * pl], py = a.pos[3 * pl + 1], pz = a.pos[3 * pl + 2];
+    const float nx = a.nrm[3 * pl], ny = a.nrm[3 * pl + 1], nz = a.nrm[3 * pl + 2];
+    xp::Pixel pp = xp::make_pixel(px, py, pz, nx, ny, nz, a.neg0, true);
+    const bool pixel_ok = pp.ok;
+    const float* vrow = a.vis + pl * k;
+    float ch = 0.0f;
+    int y = 0;
+    for (int t0 = 0; t0 < n_slots; t0 += a.tile) {
+      const int t1 = min(t0 + a.tile, n_slots);
+      if (!whole) {
+        __syncthreads();   // the previous tile is read by every thread
+        lights_ok = __syncthreads_and(stage_slots(a, s_off, s_pad, s_lt, t0, t1 - t0)) != 0;
+      }
+      pp.ok = pixel_ok && lights_ok;
+      int cur = t0;
+      while (y < k) {
+        const int pad_end = s_pad[y + 1], end = min(pad_end, t1);
+        // the run's bounds are checked once; a run that breaks them is summed
+        // again, light by light, from where it began
+        const float ch0 = ch;
+        float dmin = 1.0f;
+        uint32_t tmin = 0xFFFFFFFFu;
+#pragma unroll 2
+        for (int i = cur - t0; i < end - t0; i += 2) {
+          const float2 c = xp::contribution2(pp, s_lt[i], s_lt[i + 1], dmin, tmin);
+          ch = __fadd_rn(__fadd_rn(ch, c.x), c.y);
         }
-        const float wy = __fmul_rn(fmaxf(v, bits_f(kVisClampBits)), ch);
-#pragma unroll
-        for (int t = 0; t < kMaxClusters; ++t)
-          if (t == y) w[t] = wy;
-        wsum = __fadd_rn(wsum, wy);
-      }
-    }
-    if (!live) continue;   // the last batch: nothing to pick, no barrier follows
-    const int y = cluster_reservoir(w, k, pixel, frame, view, k0, k1);
-    int sel_light = -1;
-    float W = 0.0f, cx = 0.0f;
-    if (y >= 0) {
-      float w_y = 0.0f;
-#pragma unroll
-      for (int t = 0; t < kMaxClusters; ++t)
-        if (t == y) w_y = w[t];
-      // step 2: streaming RIS among kRis uniform members of cluster y
-      const int base = s_off[y];
-      const uint32_t m_y = (uint32_t)(s_off[y + 1] - base);
-      const uint4 u = philox4x32_10(make_uint4(pixel, frame, view, (0u << 4) | kTagRis), k0, k1);
-      const uint4 v = philox4x32_10(make_uint4(pixel, frame, view, (1u << 4) | kTagRis), k0, k1);
-      const uint32_t ru[kRis] = {u.x, u.y, u.z, u.w};
-      const uint32_t rr[kRis] = {v.x, v.y, v.z, v.w};
-      int slot[kRis];
-      float cc[kRis];
-#pragma unroll
-      for (int t = 0; t < kRis; ++t) {
-        slot[t] = base + (int)(((uint64_t)ru[t] * m_y) >> 32);
-        const float4 l = kSmemLights ? s_lt[slot[t]] : light_at<false>(s_lt, lights, mem[slot[t]]);
-        cc[t] = contribution(px, py, pz, nx, ny, nz, l.x, l.y, l.z, l.w);
-      }
-      const int j = integer_reservoir(cc, kRis, rr);
-      if (j >= 0) {
-        float sum = 0.0f;
-#pragma unroll
-        for (int t = 0; t < kRis; ++t) sum = __fadd_rn(sum, cc[t]);
-        float c_j = 0.0f;
-        int s_j = 0;
-#pragma unroll
-        for (int t = 0; t < kRis; ++t)
-          if (t == j) {
-            c_j = cc[t];
-            s_j = slot[t];
+        if (!xp::in_bounds(pp, dmin, tmin)) {
+          ch = ch0;
+#pragma unroll 1
+          for (int i = cur - t0; i < end - t0; ++i) {
+            const float4 l = xp::pair_light(s_lt, i);
+            ch = __fadd_rn(ch, contribution(px, py, pz, nx, ny, nz, l.x, l.y, l.z, l.w));
           }
-        const float mean = __fdiv_rn(sum, (float)kRis);
-        const float pr = __fdiv_rn(__fdiv_rn(w_y, wsum), (float)m_y);
-        W = __fdiv_rn(mean, __fmul_rn(pr, c_j));
-        sel_light = mem[s_j];
-        cx = c_j;
+        }
+        cur = end;
+        if (pad_end > t1) break;
+        s_w[y * kSumThreads] = __fmul_rn(fmaxf(__ldg(vrow + y), bits_f(kVisClampBits)), ch);
+        ch = 0.0f;
+        ++y;
       }
     }
-    if (light_out) light_out[p] = sel_light;
-    if (weight_out) weight_out[p] = W;
-    if (estimate) {
-      float e = 0.0f;
-      if (sel_light >= 0) {
-        const float4 l = reinterpret_cast<const float4*>(lights)[sel_light];
-        if (!segment_blocked(px, py, pz, l.x, l.y, l.z, occ)) e = __fmul_rn(cx, W);
-      }
-      estimate[p] = e;
-    }
+    if (!live) continue;   // the last batch: no barrier follows
+    float wsum = 0.0f;
+    for (int t = 0; t < k; ++t) wsum = __fadd_rn(wsum, s_w[t * kSumThreads]);
+    y = cluster_reservoir([&](int t) { return s_w[t * kSumThreads]; }, k,
+                          (uint32_t)(a.pixel_offset + p), a.frame, a.view, a.k0, a.k1);
+    const int base = y < 0 ? 0 : s_off[y];
+    pp.ok = pixel_ok;
+    finish_pixel(a, p, y, y < 0 ? 0.0f : s_w[y * kSumThreads], wsum, base,
+                 y < 0 ? 0u : (uint32_t)(s_off[y + 1] - base), px, py, pz, pp,
+                 [&](int slot) {
+                   return whole ? xp::pair_light(s_lt, s_pad[y] + slot - base) : table_light(a, slot);
+                 },
+                 occ);
   }
 }
 
@@ -435,17 +514,19 @@ cudaError_t launch_cluster_targets(const nvc_scene* sc, const nvc_clusters* cl, 
   return cudaGetLastError();
 }
 
-// Shared memory of the sampler: the occluders, plus the lights when they fit
-// in the 227 KB a block may opt into (about 14,000 lights); beyond that the
-// lights are read through the read-only cache.
-constexpr size_t kSmemOptin = 227 * 1024;
+// Light slots the sum kernel stages at once: all of them (each cluster may
+// add one to be even) up to a tile.
+static int light_slots(const nvc_scene* sc, const nvc_clusters* cl) {
+  const int64_t all = ((int64_t)sc->n_lights + cl->k + 3) & ~(int64_t)3;
+  return (int)(all < kLightTile ? all : kLightTile);
+}
 
 size_t sample_clustered_smem(const nvc_scene* sc, const nvc_clusters* cl) {
   const size_t occ =
       occluder_bytes(sc->n_spheres, sc->n_boxes) + sizeof(float4) * ((kMaxClusters + 4) / 4);
   if (cl->weights == NVC_CLUSTER_WEIGHT_VISIBILITY) return occ;   // no light loop
-  const size_t lt = sizeof(float) * 4 * (size_t)sc->n_lights;
-  return occ + lt <= kSmemOptin ? occ + lt : occ + sizeof(float4) * kLightTile;
+  return occ + sizeof(float4) * ((kMaxClusters + 4) / 4 + light_slots(sc, cl)) +
+         sizeof(float) * kMaxClusters * kSumThreads;
 }
 
 cudaError_t launch_sample_clustered(const nvc_scene* sc, const nvc_clusters* cl, const float* vis,
@@ -455,40 +536,30 @@ cudaError_t launch_sample_clustered(const nvc_scene* sc, const nvc_clusters* cl,
                                     int num_sms, cudaStream_t s) {
   if (n == 0) return cudaSuccess;
   const size_t smem = sample_clustered_smem(sc, cl);
-  const bool lights_on_chip =
-      occluder_bytes(sc->n_spheres, sc->n_boxes) + sizeof(float4) * ((kMaxClusters + 4) / 4) +
-          sizeof(float) * 4 * (size_t)sc->n_lights <=
-      kSmemOptin;
-  auto kern = cl->weights == NVC_CLUSTER_WEIGHT_VISIBILITY ? sample_clustered_kernel<false, false>
-              : lights_on_chip                             ? sample_clustered_kernel<true, true>
-                                                           : sample_clustered_kernel<false, true, true>;
+  const ClusterArgs a{sc->lights, sc->n_lights, sc->spheres, sc->n_spheres, sc->boxes, sc->n_boxes,
+                      cl->offsets, cl->members, cl->k, vis, pos, nrm, n, pixel_offset,
+                      (uint32_t)seed, (uint32_t)(seed >> 32), frame, view, light, weight, estimate,
+                      -0.0f, light_slots(sc, cl)};
+  const bool sum = cl->weights != NVC_CLUSTER_WEIGHT_VISIBILITY;
+  const void* kern = sum ? (const void*)sample_sum_kernel : (const void*)sample_visibility_kernel;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  // The staged lights are shared by a CTA's threads: take the smallest CTA
-  // (128 .. 1024 threads) that keeps the most threads resident per SM, so a
-  // large light set does not cut residency.  One wave of resident CTAs
-  // strides over the pixels.
-  int threads = 128, best = 0;
-  for (int t = 128; t <= 1024; t *= 2) {
-    int per_sm = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, t, smem);
-    if (e != cudaSuccess) return e;
-    if (per_sm * t > best) {
-      best = per_sm * t;
-      threads = t;
-    }
-  }
-  if (best == 0) return cudaErrorInvalidConfiguration;
-  const int64_t want = (n + threads - 1) / threads;
-  const int64_t cap = (int64_t)num_sms * (best / threads);
+  // one wave of resident CTAs strides over the pixels
+  const int threads = sum ? kSumThreads : 128;
+  int per_sm = 0;
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem);
+  if (e != cudaSuccess) return e;
+  if (per_sm == 0) return cudaErrorInvalidConfiguration;
+  const int64_t want = (n + threads - 1) / threads, cap = (int64_t)num_sms * per_sm;
   const int grid = (int)(want < cap ? want : cap);
-  // 16-byte loads of a pixel's visibilities need rows of a multiple of 4
-  // floats on a 16-byte aligned base
-  const bool vis_vec4 = (cl->k & 3) == 0 && (reinterpret_cast<uintptr_t>(vis) & 15) == 0;
-  kern<<<grid, threads, smem, s>>>(sc->lights, sc->n_lights, sc->spheres, sc->n_spheres, sc->boxes,
-                                   sc->n_boxes, cl->offsets, cl->members, cl->k, vis, pos, nrm, n,
-                                   pixel_offset, (uint32_t)seed, (uint32_t)(seed >> 32), frame,
-                                   view, light, weight, estimate, vis_vec4);
+  if (sum) {
+    sample_sum_kernel<<<grid, threads, smem, s>>>(a);
+  } else {
+    // 16-byte loads of a pixel's visibilities need rows of a multiple of 4
+    // floats on a 16-byte aligned base
+    sample_visibility_kernel<<<grid, threads, smem, s>>>(
+        a, (cl->k & 3) == 0 && (reinterpret_cast<uintptr_t>(vis) & 15) == 0);
+  }
   return cudaGetLastError();
 }
 

@@ -17,12 +17,14 @@
 // (same operations in the same order), so the results are theirs bit for bit.
 //
 // Measured, 1920x1080 pixels of the paper's preset (10 levels x 4 features,
-// MLP 40-32-32-32, 32 lights): 0.666 ms; as three kernels that staged
+// MLP 40-32-32-32, 32 lights): 0.611 ms; as three kernels that staged
 // features and visibilities in memory, 65,536 pixels at a time, 2.78 ms (MLP
-// 1.57, encode 0.48, sampler 0.77).  Bound by instruction issue (7,350 a
-// pixel, 59% of the slots at 16 warps an SM).
+// 1.57, encode 0.48, sampler 0.77).  Bound by instruction issue; 24 warps an
+// SM (80 registers) took 0.611 ms, 16 warps 0.625, and contributions one
+// light at a time 0.666.
 #include <cfloat>
 
+#include "exact_pair.cuh"
 #include "fp32_common.cuh"
 #include "fused_common.cuh"
 #include "hashgrid.cuh"
@@ -49,6 +51,7 @@ struct ShadeArgs {
   int L;
   uint32_t k0, k1, frame, view;
   int64_t pixel_offset;
+  float neg0;           // -0.0f (exact_pair.cuh)
   int32_t* idx;
   float* pdf;
   float* wsum;
@@ -59,19 +62,23 @@ struct ShadeArgs {
 constexpr int kWarps = 8;
 
 template <int F, bool SHADE>
-__global__ void __launch_bounds__(kWarps * 32, 2) shade_f32_kernel(const __grid_constant__ ShadeArgs a) {
+__global__ void __launch_bounds__(kWarps * 32, 3) shade_f32_kernel(const __grid_constant__ ShadeArgs a) {
   extern __shared__ __align__(16) float sm[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, n_warps = blockDim.x >> 5;
   stage_weights(a.net, a.params, sm, threadIdx.x, blockDim.x);
   float4* s_l = reinterpret_cast<float4*>(sm + a.light_off);
+  bool lights_ok = true;
   if constexpr (SHADE) {
-    for (int e = threadIdx.x; e < a.L; e += blockDim.x) {
-      float4 l = reinterpret_cast<const float4*>(a.lights)[e];
+    // in groups of four, zero lights past the last
+    for (int e = threadIdx.x; e < ((a.L + 3) & ~3); e += blockDim.x) {
+      float4 l = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (e < a.L) l = reinterpret_cast<const float4*>(a.lights)[e];
       l.w = __fmul_rn(l.w, bits_f(kInvPiBits));
-      s_l[e] = l;
+      xp::put_light(s_l, e, l);
+      lights_ok = lights_ok && xp::light_ok(l);
     }
   }
-  __syncthreads();
+  lights_ok = __syncthreads_and(lights_ok) != 0;
   float* buf = sm + a.warp_off + warp * a.warp_floats;
   const int rg = lane & 7, og = lane >> 3;   // the lane's 4 pixels and 8 outputs of 32
   const int L = a.L, last = a.net.n_layers - 1;
@@ -157,16 +164,21 @@ __global__ void __launch_bounds__(kWarps * 32, 2) shade_f32_kernel(const __grid_
         const float nx = __ldg(a.nrm + 3 * row), ny = __ldg(a.nrm + 3 * row + 1),
                     nz = __ldg(a.nrm + 3 * row + 2);
         float wmax = 0.0f, sum = 0.0f, di = 0.0f;
-#pragma unroll 2
-        for (int i = 0; i < L; ++i) {
-          const float4 l = s_l[i];
-          const float c = contribution(px, py, pz, nx, ny, nz, l.x, l.y, l.z, l.w);
-          const float vi = v[i * kLd];
-          const float wi = __fmul_rn(fmaxf(vi, bits_f(kVisClampBits)), c);
-          wmax = fmaxf(wmax, wi);
-          sum += wi;
-          di = fmaf(vi, c, di);
-          v[i * kLd] = wi;
+        const xp::Pixel pixel_pairs = xp::make_pixel(px, py, pz, nx, ny, nz, a.neg0, lights_ok);
+        for (int i0 = 0; i0 < L; i0 += 4) {
+          float c[4];
+          xp::staged_contributions<2>(pixel_pairs, s_l + i0, c);
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            if (i0 + q < L) {
+              const float vi = v[(i0 + q) * kLd];
+              const float wi = __fmul_rn(fmaxf(vi, bits_f(kVisClampBits)), c[q]);
+              wmax = fmaxf(wmax, wi);
+              sum += wi;
+              di = fmaf(vi, c[q], di);
+              v[(i0 + q) * kLd] = wi;
+            }
+          }
         }
         int sel = -1;
         const uint32_t pixel = (uint32_t)(a.pixel_offset + row);
@@ -214,7 +226,7 @@ size_t plan_smem(const nvc_handle* h, const Net& net, int warps, ShadeArgs* a) {
   const bool one = widest <= 32;
   const int area = (one ? (dims[0] > dims[1] ? dims[0] : dims[1]) : dims[0] + dims[1]) * kLd;
   const int light_off = (net.t_floats + 3) & ~3;
-  const int warp_off = light_off + 4 * ((h->L + 1) & ~1);
+  const int warp_off = light_off + 4 * ((h->L + 3) & ~3);
   if (a) {
     a->light_off = light_off;
     a->warp_off = warp_off;
@@ -261,6 +273,7 @@ ShadeArgs common_args(const nvc_handle* h, const float* pos, int64_t n) {
   a.ep = encode_params(h);
   a.net = make_net(h);
   a.L = h->L;
+  a.neg0 = -0.0f;
   return a;
 }
 
