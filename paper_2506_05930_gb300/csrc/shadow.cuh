@@ -149,31 +149,201 @@ __device__ __forceinline__ bool box_blocks_general(float px, float py, float pz,
   return !miss && tmin <= tmax;
 }
 
+// fl(1 / x): Markstein's correction of the hardware's approximate reciprocal
+// (two, the first of the reciprocal itself; exact_pair.cuh names the method,
+// and its check of every mantissa pair covers 1 / x), the library's division
+// outside [2^-60, 2^60].
+__device__ __forceinline__ float rcp_rn(float x) {
+  const float ax = fabsf(x);
+  if (!(ax >= 0x1p-60f && ax <= 0x1p60f)) return __fdiv_rn(1.0f, x);
+  float y;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  y = __fmaf_rn(__fmaf_rn(-x, y, 1.0f), y, y);
+  return __fmaf_rn(__fmaf_rn(-x, y, 1.0f), y, y);
+}
+
+// A segment from x to a light, with the reciprocals the tests share.
+struct Segment {
+  float px, py, pz, dx, dy, dz;
+  float inv_dd, ix, iy, iz;
+  bool oblique;   // no component of d is zero
+};
+
+__device__ __forceinline__ Segment make_segment(float px, float py, float pz, float lx, float ly,
+                                                float lz) {
+  Segment g;
+  g.px = px;
+  g.py = py;
+  g.pz = pz;
+  g.dx = __fsub_rn(lx, px);
+  g.dy = __fsub_rn(ly, py);
+  g.dz = __fsub_rn(lz, pz);
+  const float dd = dot3_rn(g.dx, g.dy, g.dz, g.dx, g.dy, g.dz);
+  // a zero-length segment (light on the point): t stays at t0
+  g.inv_dd = dd > 0.0f ? rcp_rn(dd) : 0.0f;
+  g.ix = g.dx != 0.0f ? rcp_rn(g.dx) : 0.0f;
+  g.iy = g.dy != 0.0f ? rcp_rn(g.dy) : 0.0f;
+  g.iz = g.dz != 0.0f ? rcp_rn(g.dz) : 0.0f;
+  g.oblique = g.dx != 0.0f && g.dy != 0.0f && g.dz != 0.0f;
+  return g;
+}
+
+// Staged sphere i (of 2 n_pairs slots) and box i against the segment.
+__device__ __forceinline__ bool sphere_blocks(const Segment& g, const Occluders& occ, int i) {
+  const float* q = reinterpret_cast<const float*>(occ.sph) + (i >> 1) * 8 + (i & 1);
+  return sphere_lane_blocks(g.px, g.py, g.pz, g.dx, g.dy, g.dz, g.inv_dd, q[0], q[2], q[4], q[6]);
+}
+
+__device__ __forceinline__ bool box_blocks(const Segment& g, const Occluders& occ, int i) {
+  const float2* b = occ.box + 3 * i;
+  if (!g.oblique)
+    return box_blocks_general(g.px, g.py, g.pz, g.dx, g.dy, g.dz, g.ix, g.iy, g.iz, b);
+  return box_blocks_oblique(make_float2(g.px, g.px), make_float2(g.py, g.py),
+                            make_float2(g.pz, g.pz), make_float2(g.ix, g.ix),
+                            make_float2(g.iy, g.iy), make_float2(g.iz, g.iz), b);
+}
+
 // Whether the segment from (px, py, pz) to the light at (lx, ly, lz) is
 // blocked by one of the staged occluders.
 __device__ __forceinline__ bool segment_blocked(float px, float py, float pz, float lx, float ly,
                                                 float lz, const Occluders& occ) {
-  const float dx = __fsub_rn(lx, px), dy = __fsub_rn(ly, py), dz = __fsub_rn(lz, pz);
-  const float dd = dot3_rn(dx, dy, dz, dx, dy, dz);
-  // a zero-length segment (light on the point): t stays at t0
-  const float inv_dd = dd > 0.0f ? __fdiv_rn(1.0f, dd) : 0.0f;
-  const float ix = dx != 0.0f ? __fdiv_rn(1.0f, dx) : 0.0f;
-  const float iy = dy != 0.0f ? __fdiv_rn(1.0f, dy) : 0.0f;
-  const float iz = dz != 0.0f ? __fdiv_rn(1.0f, dz) : 0.0f;
+  const Segment g = make_segment(px, py, pz, lx, ly, lz);
   const float2 px2 = make_float2(px, px), py2 = make_float2(py, py), pz2 = make_float2(pz, pz);
   bool blocked = false;
   for (int k = 0; k < occ.n_pairs && !blocked; ++k)
-    blocked = sphere_pair_blocks(px, py, pz, dx, dy, dz, inv_dd, occ.sph[2 * k], occ.sph[2 * k + 1]);
+    blocked = sphere_pair_blocks(px, py, pz, g.dx, g.dy, g.dz, g.inv_dd, occ.sph[2 * k],
+                                 occ.sph[2 * k + 1]);
   if (blocked) return true;
-  if (dx != 0.0f && dy != 0.0f && dz != 0.0f) {
-    const float2 ix2 = make_float2(ix, ix), iy2 = make_float2(iy, iy), iz2 = make_float2(iz, iz);
+  if (g.oblique) {
+    const float2 ix2 = make_float2(g.ix, g.ix), iy2 = make_float2(g.iy, g.iy),
+                 iz2 = make_float2(g.iz, g.iz);
     for (int k = 0; k < occ.n_box && !blocked; ++k)
       blocked = box_blocks_oblique(px2, py2, pz2, ix2, iy2, iz2, occ.box + 3 * k);
   } else {
     for (int k = 0; k < occ.n_box && !blocked; ++k)
-      blocked = box_blocks_general(px, py, pz, dx, dy, dz, ix, iy, iz, occ.box + 3 * k);
+      blocked = box_blocks_general(px, py, pz, g.dx, g.dy, g.dz, g.ix, g.iy, g.iz, occ.box + 3 * k);
   }
   return blocked;
+}
+
+// ---- a warp's segments together ------------------------------------------------
+// 32 neighbouring pixels looking at one light sweep a thin volume that most
+// occluders are nowhere near.  Each lane holds a different occluder against
+// that volume -- the pixels' bounding box moved along the segment from its
+// centre to the light -- and only the occluders whose vote stands are tested
+// exactly, by all lanes, each against its own segment.
+//
+// The vote never drops an occluder that an exact test would call blocking:
+// every segment lies in the swept box, so the occluder is held against it
+// grown by 2^-16 of the largest coordinate involved, 16 times and more what
+// the exact tests' roundings (some 2^-20 of it) and the vote's own can add
+// up to; and it is written so that anything not a number stands.
+struct WarpHull {
+  float cx, cy, cz;   // centre and half extents of the 32 positions
+  float hx, hy, hz;
+  float rad;          // |half extents|, rounded up
+  float scale;        // largest coordinate magnitude
+};
+
+__device__ __forceinline__ WarpHull warp_hull(float px, float py, float pz) {
+  float lo[3] = {px, py, pz}, hi[3] = {px, py, pz};
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      lo[a] = fminf(lo[a], __shfl_xor_sync(0xffffffffu, lo[a], o));
+      hi[a] = fmaxf(hi[a], __shfl_xor_sync(0xffffffffu, hi[a], o));
+    }
+  WarpHull w;
+  w.cx = 0.5f * (lo[0] + hi[0]);
+  w.cy = 0.5f * (lo[1] + hi[1]);
+  w.cz = 0.5f * (lo[2] + hi[2]);
+  w.hx = 0.5f * (hi[0] - lo[0]);
+  w.hy = 0.5f * (hi[1] - lo[1]);
+  w.hz = 0.5f * (hi[2] - lo[2]);
+  w.rad = 1.0001f * sqrtf(w.hx * w.hx + w.hy * w.hy + w.hz * w.hz);
+  w.scale = fmaxf(fmaxf(fabsf(w.cx) + w.hx, fabsf(w.cy) + w.hy), fabsf(w.cz) + w.hz);
+  return w;
+}
+
+// Whether the lane's segments' volume may meet staged sphere i / box i.
+struct HullRay {
+  float dx, dy, dz;      // light - centre
+  float inv_dd, ix, iy, iz;
+  float scale;
+};
+
+__device__ __forceinline__ HullRay hull_ray(const WarpHull& w, float lx, float ly, float lz) {
+  HullRay r;
+  r.dx = lx - w.cx;
+  r.dy = ly - w.cy;
+  r.dz = lz - w.cz;
+  const float dd = r.dx * r.dx + r.dy * r.dy + r.dz * r.dz;
+  r.inv_dd = dd > 0.0f ? __fdividef(1.0f, dd) : 0.0f;
+  // a component of zero: as good as zero, but with a finite reciprocal
+  r.ix = __fdividef(1.0f, copysignf(fmaxf(fabsf(r.dx), 1e-20f), r.dx));
+  r.iy = __fdividef(1.0f, copysignf(fmaxf(fabsf(r.dy), 1e-20f), r.dy));
+  r.iz = __fdividef(1.0f, copysignf(fmaxf(fabsf(r.dz), 1e-20f), r.dz));
+  r.scale = w.scale + fmaxf(fmaxf(fabsf(lx), fabsf(ly)), fabsf(lz));
+  return r;
+}
+
+__device__ __forceinline__ bool hull_meets_sphere(const WarpHull& w, const HullRay& r,
+                                                  const Occluders& occ, int i) {
+  const float* q = reinterpret_cast<const float*>(occ.sph) + (i >> 1) * 8 + (i & 1);
+  const float sx = q[0], sy = q[2], sz = q[4], r2 = q[6];
+  const float ox = sx - w.cx, oy = sy - w.cy, oz = sz - w.cz;
+  const float t = fminf(fmaxf((ox * r.dx + oy * r.dy + oz * r.dz) * r.inv_dd, 0.0f), 1.0f);
+  const float ex = ox - t * r.dx, ey = oy - t * r.dy, ez = oz - t * r.dz;
+  const float m = 0x1p-16f * (r.scale + fmaxf(fmaxf(fabsf(sx), fabsf(sy)), fabsf(sz)));
+  const float reach = 1.0001f * sqrtf(r2) + w.rad + m;
+  return r2 >= 0.0f && !(ex * ex + ey * ey + ez * ez > reach * reach);
+}
+
+__device__ __forceinline__ bool hull_meets_box(const WarpHull& w, const HullRay& r,
+                                               const Occluders& occ, int i) {
+  const float2 bx = occ.box[3 * i], by = occ.box[3 * i + 1], bz = occ.box[3 * i + 2];
+  const float m = 0x1p-16f * (r.scale + fmaxf(fmaxf(fmaxf(fabsf(bx.x), fabsf(bx.y)),
+                                                   fmaxf(fabsf(by.x), fabsf(by.y))),
+                                             fmaxf(fabsf(bz.x), fabsf(bz.y))));
+  const float ax = (fminf(bx.x, bx.y) - w.hx - m - w.cx) * r.ix,
+              cx = (fmaxf(bx.x, bx.y) + w.hx + m - w.cx) * r.ix;
+  const float ay = (fminf(by.x, by.y) - w.hy - m - w.cy) * r.iy,
+              cy = (fmaxf(by.x, by.y) + w.hy + m - w.cy) * r.iy;
+  const float az = (fminf(bz.x, bz.y) - w.hz - m - w.cz) * r.iz,
+              cz = (fmaxf(bz.x, bz.y) + w.hz + m - w.cz) * r.iz;
+  const float tmin = fmaxf(fmaxf(fminf(ax, cx), fminf(ay, cy)), fmaxf(fminf(az, cz), 0.0f));
+  const float tmax = fminf(fminf(fmaxf(ax, cx), fmaxf(ay, cy)), fminf(fmaxf(az, cz), 1.0f));
+  return !(tmin > tmax);
+}
+
+// segment_blocked for a whole warp looking at one light: the lanes with
+// `want` get their answer, the others false.  *tested (the same in all lanes)
+// grows by the exact tests taken.
+__device__ __forceinline__ bool warp_segments_blocked(const WarpHull& w, bool want, float px, float py,
+                                                      float pz, float lx, float ly, float lz,
+                                                      const Occluders& occ, int* tested) {
+  const int lane = threadIdx.x & 31;
+  const HullRay r = hull_ray(w, lx, ly, lz);
+  const Segment g = make_segment(px, py, pz, lx, ly, lz);
+  bool open = want;
+  for (int b = 0; b < 2 * occ.n_pairs; b += 32) {
+    const bool near = b + lane < 2 * occ.n_pairs && hull_meets_sphere(w, r, occ, b + lane);
+    for (unsigned m = __ballot_sync(0xffffffffu, near); m; m &= m - 1) {
+      open = open && !sphere_blocks(g, occ, b + __ffs(m) - 1);
+      ++*tested;
+      if (!__any_sync(0xffffffffu, open)) return want;
+    }
+  }
+  for (int b = 0; b < occ.n_box; b += 32) {
+    const bool near = b + lane < occ.n_box && hull_meets_box(w, r, occ, b + lane);
+    for (unsigned m = __ballot_sync(0xffffffffu, near); m; m &= m - 1) {
+      open = open && !box_blocks(g, occ, b + __ffs(m) - 1);
+      ++*tested;
+      if (!__any_sync(0xffffffffu, open)) return want;
+    }
+  }
+  return want && !open;
 }
 
 // ---- training positions (Section 3.4) ------------------------------------------

@@ -78,6 +78,23 @@ def _same(a, b):
     return torch.equal(torch.nan_to_num(a, nan=-7.0), torch.nan_to_num(b, nan=-7.0))
 
 
+@pytest.mark.parametrize("kind", ["line", "random", "odd"])
+@pytest.mark.parametrize("n,L,ns,nb", [(1, 1, 0, 0), (31, 3, 1, 0), (33, 4, 0, 1), (64, 9, 33, 31),
+                                       (1000, 32, 32, 32), (257, 37, 65, 70), (300, 15000, 3, 2)])
+def test_exact_di_equals_one_light_at_a_time(kind, n, L, ns, nb):
+    from paper_2506_05930_gb300 import nvc
+    pos, nrm = _pixels(kind, n, seed=n)
+    lights = _lights(kind, L, pos, seed=L)
+    P, N = torch.from_numpy(pos).cuda(), torch.from_numpy(nrm).cuda()
+    c, v = _per_light(lights, ns, nb, n, P, N)
+    ref = torch.zeros(n, device="cuda")
+    for i in range(L):
+        ref = torch.where((c[:, i] > 0) & (v[:, i] > 0), ref + c[:, i], ref)
+    di = torch.empty(n, device="cuda")
+    nvc.nvc_exact_di(_scene(lights, ns, nb, n), P, N, di)
+    assert _same(di, ref)
+
+
 @pytest.mark.parametrize("kind", ["line", "odd"])
 @pytest.mark.parametrize("n,L,k", [(1, 1, 1), (33, 7, 3), (300, 37, 32), (700, 1021, 31),
                                    (500, 1025, 8), (70, 5000, 5)])
