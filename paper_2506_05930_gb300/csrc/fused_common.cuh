@@ -240,12 +240,13 @@ __device__ __forceinline__ float2 contribution2_fast(float2 npx, float2 npy, flo
   return c;
 }
 
+__host__ __device__ __forceinline__ int round_up16(int x) { return (x + 15) & ~15; }
+
 // Stages the L lights (float4 x, y, z, I) as pairs for contribution2_fast,
-// I scaled by 1/pi; an odd count's last slot is zero.  Threads t of
-// nthreads share the work; the caller synchronises.
+// I scaled by 1/pi; slots from L to Lp (an even count) are zero lights.
+// Threads t of nthreads share the work; the caller synchronises.
 __device__ __forceinline__ void stage_light_pairs(float4* s_pairs, const float* lights, int L,
-                                                  int t, int nthreads) {
-  const int Lp = (L + 1) & ~1;
+                                                  int t, int nthreads, int Lp) {
   for (int e = t; e < Lp; e += nthreads) {
     float4 l = e < L ? reinterpret_cast<const float4*>(lights)[e] : make_float4(0.f, 0.f, 0.f, 0.f);
     l.w = __fmul_rn(l.w, bits_f(kInvPiBits));

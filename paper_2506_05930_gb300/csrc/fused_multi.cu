@@ -81,7 +81,7 @@ __global__ void __launch_bounds__(kTileM * TPC, TPC == 2 ? 3 : 2)
 
   for (int e = t; e < a.wimg_bytes / 16; e += kThreads)
     reinterpret_cast<uint4*>(s_w)[e] = a.wimg[e];
-  if (a.lights) stage_light_pairs(s_l, a.lights, a.L, t, kThreads);
+  if (a.lights) stage_light_pairs(s_l, a.lights, a.L, t, kThreads, (a.L + 1) & ~1);
   if (t == 0) {
     for (int gg = 0; gg < TPC; ++gg) mbar_init(smem_u32(s_bar + gg), 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");

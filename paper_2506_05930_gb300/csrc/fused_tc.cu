@@ -54,7 +54,7 @@ __global__ void __launch_bounds__(kTileM, 5) fused_shade_kernel(const __grid_con
 
   for (int e = t; e < a.wimg_bytes / 16; e += kTileM)
     reinterpret_cast<uint4*>(s_w)[e] = a.wimg[e];
-  if (a.lights) stage_light_pairs(s_l, a.lights, a.L, t, kTileM);
+  if (a.lights) stage_light_pairs(s_l, a.lights, a.L, t, kTileM, (a.L + 1) & ~1);
   const uint32_t bar = smem_u32(s_bar);
   if (t == 0) {
     mbar_init(bar, 1);
@@ -328,6 +328,15 @@ __global__ void __launch_bounds__(kTileM, 5) fused_shade_kernel(const __grid_con
 // Sum w and Neural DI are the first half's sum plus the second half's, so
 // they can differ from the other variants' one-pass sums in the last bits;
 // the picks are the same integers from the same float32 weights.
+//
+// The light table is padded to whole 16-light chunks with zero lights, whose
+// weight is 0 whatever the padded logit says, so the sampler's loops carry no
+// bounds: with a bound per light the compiler kept a compare and a predicate
+// on every operation.  3840x2160 x 256 lights, FP16: 6.87 -> 5.03 ms; four
+// views of 128 lights (14,976,000 random points): 7.97 -> 7.75 ms, there with
+// half the time in the encode's scattered row reads.  Four threads per pixel
+// (32 warps an SM where the accumulators' TMEM columns leave 16) took 5.39
+// and 9.62 ms: the pipes, not the warps in flight, are what is short.
 // (constant barrier ids, so the CTA holds five hardware barriers, not 16)
 __device__ __forceinline__ void pair_sync(int warp) {
   switch (warp & 3) {
@@ -358,7 +367,7 @@ __global__ void __launch_bounds__(2 * kTileM, 3) fused_shade_pair_kernel(const _
 
   for (int e = t; e < a.wimg_bytes / 16; e += kThreads)
     reinterpret_cast<uint4*>(s_w)[e] = a.wimg[e];
-  if (a.lights) stage_light_pairs(s_l, a.lights, a.L, t, kThreads);
+  if (a.lights) stage_light_pairs(s_l, a.lights, a.L, t, kThreads, round_up16(a.L));
   const uint32_t bar = smem_u32(s_bar);
   if (t == 0) {
     mbar_init(bar, 1);
@@ -397,9 +406,10 @@ __global__ void __launch_bounds__(2 * kTileM, 3) fused_shade_pair_kernel(const _
   const int K0 = a.layer[0].K;
   const int64_t n_tiles = a.n_tiles;
   const int L = a.L;
-  const int H = split_h(L);   // first half: lights [0, H)
+  const int L16 = round_up16(L);   // whole chunks
+  const int H = split_h(L);        // first half: lights [0, H)
   const int lo = half ? H : 0;
-  const int hi = half ? L : (H < L ? H : L);
+  const int hi = half ? L16 : (H < L16 ? H : L16);
 
   for (int64_t tile = *s_next; tile < n_tiles && !failed; tile = *s_next) {
     const ViewDesc& V = a.v[view_of(a, tile)];
@@ -498,7 +508,7 @@ __global__ void __launch_bounds__(2 * kTileM, 3) fused_shade_pair_kernel(const _
         for (int c0 = lo; c0 < hi; c0 += 16) {
           uint32_t r[16];
           tmem_ld16(t_lane + (uint32_t)c0, r);
-          if (live) store_sigmoid_row<16>(V.vis_out + row * L + c0, r, hi - c0, outmul);
+          if (live) store_sigmoid_row<16>(V.vis_out + row * L + c0, r, L - c0, outmul);
         }
       } else {
         float nx = 0.f, ny = 0.f, nz = 0.f;
@@ -519,31 +529,24 @@ __global__ void __launch_bounds__(2 * kTileM, 3) fused_shade_pair_kernel(const _
 #pragma unroll
           for (int j = 0; j < 16; j += 2) {
             const int i = c0 + j;
-            wreg[j] = 0.0f;
-            wreg[j + 1] = 0.0f;
-            if (i < hi) {
-              const float2 c = contribution2_fast(npx, npy, npz, nx2, ny2, nz2, s_l[i], s_l[i + 1]);
-              float2 z01 = make_float2(__uint_as_float(r[j]), __uint_as_float(r[j + 1]));
-              if constexpr (kF8) z01 = __fmul2_rn(z01, make_float2(outmul, outmul));
-              const float2 v01 = sigmoid2_fast(z01);
-              const float w0 = __fmul_rn(fmaxf(v01.x, bits_f(kVisClampBits)), c.x);
-              wmax = fmaxf(wmax, w0);
-              sum += w0;
-              di = fmaf(v01.x, c.x, di);
-              wreg[j] = w0;
-              if (i + 1 < hi) {
-                const float w1 = __fmul_rn(fmaxf(v01.y, bits_f(kVisClampBits)), c.y);
-                wmax = fmaxf(wmax, w1);
-                sum += w1;
-                di = fmaf(v01.y, c.y, di);
-                wreg[j + 1] = w1;
-              }
-            }
+            const float2 c = contribution2_fast(npx, npy, npz, nx2, ny2, nz2, s_l[i], s_l[i + 1]);
+            float2 z01 = make_float2(__uint_as_float(r[j]), __uint_as_float(r[j + 1]));
+            if constexpr (kF8) z01 = __fmul2_rn(z01, make_float2(outmul, outmul));
+            const float2 v01 = sigmoid2_fast(z01);
+            const float2 w2 = __fmul2_rn(make_float2(fmaxf(v01.x, bits_f(kVisClampBits)),
+                                                     fmaxf(v01.y, bits_f(kVisClampBits))), c);
+            wmax = fmaxf(fmaxf(wmax, w2.x), w2.y);
+            sum += w2.x;
+            di = fmaf(v01.x, c.x, di);
+            sum += w2.y;
+            di = fmaf(v01.y, c.y, di);
+            wreg[j] = w2.x;
+            wreg[j + 1] = w2.y;
           }
           if (V.w_out != nullptr && live) {
 #pragma unroll
             for (int j = 0; j < 16; ++j)
-              if (c0 + j < hi) V.w_out[row * L + c0 + j] = wreg[j];
+              if (c0 + j < L) V.w_out[row * L + c0 + j] = wreg[j];
           }
           if (!HSMALL) {
             // the weights replace their logits in this half's (now read)
@@ -579,7 +582,7 @@ __global__ void __launch_bounds__(2 * kTileM, 3) fused_shade_pair_kernel(const _
         // half h quantizes the first half's chunks h, h + 2, ...
         uint32_t Q = 0;
         if (!HSMALL) {
-          const int hiA = H < L ? H : L;
+          const int hiA = H < L16 ? H : L16;
           uint32_t part = 0;
           for (int c0 = half * 16; c0 < hiA; c0 += 32) {
             uint32_t r[16];
@@ -587,27 +590,15 @@ __global__ void __launch_bounds__(2 * kTileM, 3) fused_shade_pair_kernel(const _
             if (active) {
 #pragma unroll
               for (int j = 0; j < 16; ++j)
-                if (c0 + j < hiA)
-                  part += quantize_scaled(__fmul_rn(__uint_as_float(r[j]), qs.pre), qs.scale);
+                part += quantize_scaled(__fmul_rn(__uint_as_float(r[j]), qs.pre), qs.scale);
             }
           }
           s_q[half * kTileM + rw] = part;
         } else if (half == 0) {
           uint32_t QA = 0;
-          for (int c0 = lo; c0 < hi; c0 += 16) {
-            uint32_t r[16];
-            if (!HSMALL) tmem_ld16(t_lane + (uint32_t)c0, r);
-            if (active) {
+          if (active) {
 #pragma unroll
-              for (int j = 0; j < 16; ++j) {
-                const int i = c0 + j;
-                if (i < hi) {
-                  float w = wreg[j];
-                  if (!HSMALL) w = __fmul_rn(__uint_as_float(r[j]), qs.pre);
-                  QA += quantize_scaled(w, qs.scale);
-                }
-              }
-            }
+            for (int j = 0; j < 16; ++j) QA += quantize_scaled(wreg[j], qs.scale);
           }
           s_q[rw] = QA;
         }
@@ -625,19 +616,17 @@ __global__ void __launch_bounds__(2 * kTileM, 3) fused_shade_pair_kernel(const _
 #pragma unroll
             for (int j = 0; j < 16; ++j) {
               const int i = c0 + j;
-              if (i < hi) {
-                float w = wreg[j];
-                if (!HSMALL) w = __fmul_rn(__uint_as_float(r[j]), qs.pre);
-                if ((i & 3) == 0)
-                  rr = philox_keyed(make_uint4(pixel, a.frame, V.view,
-                                               ((uint32_t)(i >> 2) << 4) | kTagWrs),
-                                    a.rkey);
-                const uint32_t q = quantize_scaled(w, qs.scale);
-                Q += q;
-                if (__umulhi(pick_word(rr, i & 3), Q) < q) {
-                  sel = i;
-                  wsel = w;
-                }
+              float w = wreg[j];
+              if (!HSMALL) w = __fmul_rn(__uint_as_float(r[j]), qs.pre);
+              if ((j & 3) == 0)
+                rr = philox_keyed(make_uint4(pixel, a.frame, V.view,
+                                             ((uint32_t)(i >> 2) << 4) | kTagWrs),
+                                  a.rkey);
+              const uint32_t q = quantize_scaled(w, qs.scale);
+              Q += q;
+              if (__umulhi(pick_word(rr, j & 3), Q) < q) {
+                sel = i;
+                wsel = w;
               }
             }
           }
@@ -1061,7 +1050,7 @@ size_t fused_smem(const nvc_handle* h, const PackArgs& p, FusedArgs* a = nullptr
   off += (size_t)kTileM * kmax * p.esize;
   off = (off + 15) & ~(size_t)15;
   const size_t l_off = off;
-  off += 16 * (size_t)(h->L > 0 ? ((h->L + 1) & ~1) : 2);   // lights in pairs
+  off += 16 * (size_t)round_up16(h->L > 0 ? h->L : 1);   // lights in pairs
   const size_t bar_off = off;
   off += 64;
   if (a) {
