@@ -89,7 +89,7 @@ struct FusedArgs {
 // CH), zero beyond the real inputs or for a dead pixel.  TT is the table's
 // element type (float32 master or half-precision copy); the fused kernels
 // branch on it once per tile, not per level.
-template <int F, bool XSMALL, int CH, typename TT>
+template <int F, bool XSMALL, int CH, bool PAIRS = false, typename TT>
 __device__ __forceinline__ void encode_chunk(const EncodeParams& ep, const TT* table, int c,
                                              int din, float x, float y, float z, bool live,
                                              float (&fv)[CH]) {
@@ -104,7 +104,7 @@ __device__ __forceinline__ void encode_chunk(const EncodeParams& ep, const TT* t
         const int l = c * LPC + q;
         if ((l + 1) * F < din) {
           float acc[4];
-          encode_two_levels_h2<XSMALL>(ep, table, l, x, y, z, acc);
+          encode_two_levels_h2<XSMALL, PAIRS>(ep, table, l, x, y, z, acc);
 #pragma unroll
           for (int f = 0; f < 4; ++f) fv[q * F + f] = acc[f];
         } else if (l * F < din) {
@@ -123,7 +123,7 @@ __device__ __forceinline__ void encode_chunk(const EncodeParams& ep, const TT* t
       const int l = c * LPC + q;
       if (l * F < din) {
         float acc[F];
-        encode_level<F, XSMALL, true, TT>(ep, table, l, x, y, z, acc);
+        encode_level<F, XSMALL, true, TT, PAIRS>(ep, table, l, x, y, z, acc);
 #pragma unroll
         for (int f = 0; f < F; ++f) fv[q * F + f] = acc[f];
       }

@@ -334,7 +334,7 @@ __global__ void __launch_bounds__(kTileM, 5) fused_shade_kernel(const __grid_con
 // bounds: with a bound per light the compiler kept a compare and a predicate
 // on every operation.  3840x2160 x 256 lights, FP16: 6.87 -> 5.03 ms; four
 // views of 128 lights (14,976,000 random points): 7.97 -> 7.75 ms, there with
-// half the time in the encode's scattered row reads.  Four threads per pixel
+// half the time in the encode's scattered row reads (load_x_pairs).  Four threads per pixel
 // (32 warps an SM where the accumulators' TMEM columns leave 16) took 5.39
 // and 9.62 ms: the pipes, not the warps in flight, are what is short.
 // (constant barrier ids, so the CTA holds five hardware barriers, not 16)
@@ -347,8 +347,10 @@ __device__ __forceinline__ void pair_sync(int warp) {
   }
 }
 
-template <int F, int PREC, bool HSMALL>
-__global__ void __launch_bounds__(2 * kTileM, 3) fused_shade_pair_kernel(const __grid_constant__ FusedArgs a) {
+// MINB: CTAs per SM its registers leave room for; two above 128 lights, where
+// TMEM takes no more (at three, 80 registers a thread, the sampler spills).
+template <int F, int PREC, bool HSMALL, int MINB>
+__global__ void __launch_bounds__(2 * kTileM, MINB) fused_shade_pair_kernel(const __grid_constant__ FusedArgs a) {
   constexpr int kThreads = 2 * kTileM;
   extern __shared__ __align__(1024) uint8_t smem[];
   uint8_t* s_w = smem;
@@ -426,18 +428,24 @@ __global__ void __launch_bounds__(2 * kTileM, 3) fused_shade_pair_kernel(const _
       const float x = normalise(px, a.ep.lo[0], a.ep.ext[0]);
       const float y = normalise(py, a.ep.lo[1], a.ep.ext[1]);
       const float z = normalise(pz, a.ep.lo[2], a.ep.ext[2]);
-      auto encode_half = [&](const auto* tab) {
+      auto encode_half = [&](const auto* tab, auto pairs) {
         for (int c = half; c < K0 / CH; c += 2) {
           float fv[CH];
-          encode_chunk<F, false, CH>(a.ep, tab, c, din, x, y, z, live, fv);
+          encode_chunk<F, false, CH, decltype(pairs)::value>(a.ep, tab, c, din, x, y, z, live, fv);
           *reinterpret_cast<uint4*>(s_a + cm_offset(rw, c * CH, K0, ES)) =
               pack_chunk<PREC, CH>(fv, s_in0);
         }
       };
-      if (a.table16)
-        encode_half(a.table16);
-      else
-        encode_half(a.table);
+      if (F == 2 && scattered_warp(x, y, z)) {
+        if (a.table16)
+          encode_half(a.table16, std::true_type{});
+        else
+          encode_half(a.table, std::true_type{});
+      } else if (a.table16) {
+        encode_half(a.table16, std::false_type{});
+      } else {
+        encode_half(a.table, std::false_type{});
+      }
     }
     fence_async_smem();
     tc_fence_before();
@@ -1073,7 +1081,9 @@ size_t pair_smem(const nvc_handle* h, const PackArgs& p, FusedArgs* a = nullptr)
 template <int F, int PREC>
 cudaError_t launch_pair_typed(const FusedArgs& a, size_t smem_needed, int num_sms, cudaStream_t s) {
   const int H = split_h(a.L);
-  auto kern = H <= 16 ? fused_shade_pair_kernel<F, PREC, true> : fused_shade_pair_kernel<F, PREC, false>;
+  auto kern = H <= 16             ? fused_shade_pair_kernel<F, PREC, true, 3>
+              : a.tmem_cols > 128 ? fused_shade_pair_kernel<F, PREC, false, 2>
+                                  : fused_shade_pair_kernel<F, PREC, false, 3>;
   const int max_ctas = (int)(512u / a.tmem_cols);
   size_t smem = smem_needed;
   cudaFuncAttributes fa{};

@@ -286,6 +286,19 @@ __device__ __forceinline__ LevelCell level_cell(const EncodeParams& ep, int l, f
   return c;
 }
 
+// Whether a warp's pixels are not neighbours: their normalised positions (in
+// [0, 1]) spread over more than 1/8 of the domain along an axis.  32 pixels of
+// a scanline span a few hundredths, 32 positions drawn at random nearly all.
+__device__ __forceinline__ bool scattered_warp(float x, float y, float z) {
+  const uint32_t c[3] = {__float_as_uint(x), __float_as_uint(y), __float_as_uint(z)};
+  float spread = 0.0f;
+#pragma unroll
+  for (int a = 0; a < 3; ++a)
+    spread = fmaxf(spread, __uint_as_float(__reduce_max_sync(0xffffffffu, c[a])) -
+                               __uint_as_float(__reduce_min_sync(0xffffffffu, c[a])));
+  return spread > 0.125f;
+}
+
 // Packed linear interpolation of 8 corners' feature pairs (f, f + 1):
 // v0 + f (v1 - v0) along x, then y, then z.
 __device__ __forceinline__ float2 lerp_corners(const float2 (&v)[8], float fx, float fy, float fz) {
@@ -298,14 +311,69 @@ __device__ __forceinline__ float2 lerp_corners(const float2 (&v)[8], float fx, f
   return __ffma2_rn(fz2, fsub2(e1, e0), e0);
 }
 
-template <int F, bool XSMALL = false, bool LERP = true, typename TT = float>
+// The 8 corner rows of a cell from a two-feature table by x-pairs.  The x
+// prime is 1, so for an even cell x the rows of the corners x and x + 1 are
+// the two rows of one aligned pair: one load of two rows serves both, and
+// only odd cells load the second corner by itself -- 6 requests a level on
+// average instead of 8.  Each request of a lane whose neighbours are
+// elsewhere takes a cycle of the L1's tag stage, which is what an encode of
+// scattered positions is short of (four views of random points, 128 lights:
+// 7.75 -> 7.40 ms); neighbouring pixels share their requests anyway and only
+// pay the selects (10% of a 21-light frame's time).
+__device__ __forceinline__ void load_x_pairs(const float* __restrict__ tab, const uint32_t (&row)[8],
+                                             FeatVec<2> (&v)[8]) {
+  const bool joined = (row[0] ^ row[1]) == 1u;
+  float4 w[4];
+  float2 u[4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) w[k] = __ldg(reinterpret_cast<const float4*>(tab) + (row[2 * k] >> 1));
+  if (!joined) {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) u[k] = __ldg(reinterpret_cast<const float2*>(tab) + row[2 * k + 1]);
+  }
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const bool up = row[2 * k] & 1u;
+    v[2 * k].v[0] = up ? w[k].z : w[k].x;
+    v[2 * k].v[1] = up ? w[k].w : w[k].y;
+    v[2 * k + 1].v[0] = joined ? (up ? w[k].x : w[k].z) : u[k].x;
+    v[2 * k + 1].v[1] = joined ? (up ? w[k].y : w[k].w) : u[k].y;
+  }
+}
+
+// The same from a half-precision table, rows as packed half2 words.
+__device__ __forceinline__ void load_x_pairs(const unsigned int* __restrict__ tab,
+                                             const uint32_t (&row)[8], uint32_t (&v)[8]) {
+  const bool joined = (row[0] ^ row[1]) == 1u;
+  uint2 w[4];
+  uint32_t u[4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) w[k] = __ldg(reinterpret_cast<const uint2*>(tab) + (row[2 * k] >> 1));
+  if (!joined) {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) u[k] = __ldg(tab + row[2 * k + 1]);
+  }
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const bool up = row[2 * k] & 1u;
+    v[2 * k] = up ? w[k].y : w[k].x;
+    v[2 * k + 1] = joined ? (up ? w[k].x : w[k].y) : u[k];
+  }
+}
+
+// PAIRS: rows by load_x_pairs (two float32 features).
+template <int F, bool XSMALL = false, bool LERP = true, typename TT = float, bool PAIRS = false>
 __device__ __forceinline__ void encode_level(const EncodeParams& ep, const TT* __restrict__ table,
                                              int l, float x, float y, float z, float (&acc)[F]) {
   const LevelCell c = level_cell<XSMALL>(ep, l, x, y, z);
   const TT* tab = table + ((size_t)l << ep.log2_table) * F;
   FeatVec<F> v[8];
+  if constexpr (PAIRS && F == 2 && sizeof(TT) == 4) {
+    load_x_pairs(tab, c.row, v);
+  } else {
 #pragma unroll
-  for (int d = 0; d < 8; ++d) v[d] = load_row<F>(tab + (size_t)c.row[d] * F);
+    for (int d = 0; d < 8; ++d) v[d] = load_row<F>(tab + (size_t)c.row[d] * F);
+  }
   if constexpr (LERP && F % 2 == 0) {
 #pragma unroll
     for (int f = 0; f < F; f += 2) {
@@ -335,7 +403,7 @@ __device__ __forceinline__ void encode_level(const EncodeParams& ep, const TT* _
 // loads are in flight.  The rows stay packed half2 words (one register a
 // corner) until the blend widens them.  Same results as two encode_level
 // calls.
-template <bool XSMALL>
+template <bool XSMALL, bool PAIRS = false>
 __device__ __forceinline__ void encode_two_levels_h2(const EncodeParams& ep,
                                                      const __half* __restrict__ table, int la,
                                                      float x, float y, float z, float (&acc)[4]) {
@@ -344,10 +412,15 @@ __device__ __forceinline__ void encode_two_levels_h2(const EncodeParams& ep,
   const unsigned int* ta = reinterpret_cast<const unsigned int*>(table) + ((size_t)la << ep.log2_table);
   const unsigned int* tb = ta + ((size_t)1 << ep.log2_table);
   uint32_t ua[8], ub[8];
+  if constexpr (PAIRS) {
+    load_x_pairs(ta, ca.row, ua);
+    load_x_pairs(tb, cb.row, ub);
+  } else {
 #pragma unroll
-  for (int d = 0; d < 8; ++d) ua[d] = __ldg(ta + ca.row[d]);
+    for (int d = 0; d < 8; ++d) ua[d] = __ldg(ta + ca.row[d]);
 #pragma unroll
-  for (int d = 0; d < 8; ++d) ub[d] = __ldg(tb + cb.row[d]);
+    for (int d = 0; d < 8; ++d) ub[d] = __ldg(tb + cb.row[d]);
+  }
   float2 va[8], vb[8];
 #pragma unroll
   for (int d = 0; d < 8; ++d) va[d] = h2f2(ua[d]);
