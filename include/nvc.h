@@ -289,7 +289,8 @@ nvc_status nvc_calibrate(nvc_handle* h, const float* pos, int64_t n, void* strea
  * picks from the same float32 weights; all but 5 give bit-identical
  * outputs, 5 sums w and the Neural DI terms over lights [0, H) and [H, L)
  * separately (H = ceil(ceil(L / 2) / 16) * 16), which can change the last
- * bits of wsum, pdf and radiance. */
+ * bits of wsum, pdf and radiance.  A handle on which none was chosen (by the
+ * calls below) takes 0, 5 or 6 by its light and pixel count. */
 #define NVC_SHADE_VARIANTS 8
 
 /* Chooses the fused-kernel variant that nvc_infer runs (the variants give

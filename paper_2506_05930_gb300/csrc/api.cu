@@ -514,10 +514,15 @@ nvc_status nvc_infer(nvc_handle* h, const float* pos, int64_t n, float* vis, voi
     std::string why;
     if (!fused_supported(h, &why)) return fail(h, NVC_ERR_UNSUPPORTED, "%s", why.c_str());
     const int keep = h->shade_variant;
-    if (h->infer_variant >= 0) h->shade_variant = h->infer_variant;
+    const bool keep_chosen = h->variant_chosen;
+    if (h->infer_variant >= 0) {
+      h->shade_variant = h->infer_variant;
+      h->variant_chosen = true;
+    }
     const cudaError_t e = launch_shade_fused(h, nullptr, pos, nullptr, n, 0, 0, 0, 0, nullptr,
                                              nullptr, nullptr, nullptr, vis, s);
     h->shade_variant = keep;
+    h->variant_chosen = keep_chosen;
     NVC_CUDA(h, e);
     count_launches(h, 1);
     return NVC_OK;
@@ -734,6 +739,7 @@ nvc_status nvc_set_shade_plan(nvc_handle* h, const nvc_shade_plan* plan) {
   if (plan->ctas_per_sm < 0 || plan->ctas_per_sm > 64)
     return fail(h, NVC_ERR_INVALID_ARG, "ctas_per_sm out of range");
   h->shade_variant = plan->variant;
+  h->variant_chosen = true;
   h->shade_ctas_per_sm = plan->ctas_per_sm;
   return NVC_OK;
 }
@@ -753,6 +759,8 @@ nvc_status nvc_autotune_shade_plan(nvc_handle* h, const nvc_scene* scene, const 
   NVC_CUDA(h, cudaEventCreate(&e0));
   NVC_CUDA(h, cudaEventCreate(&e1));
   const int keep_v = h->shade_variant, keep_c = h->shade_ctas_per_sm;
+  const bool keep_chosen = h->variant_chosen;
+  h->variant_chosen = true;
   nvc_shade_plan best{keep_v, keep_c};
   double best_ms = -1.0;
   int np = 0;
@@ -792,6 +800,7 @@ nvc_status nvc_autotune_shade_plan(nvc_handle* h, const nvc_scene* scene, const 
   cudaEventDestroy(e1);
   if (err != cudaSuccess) {
     h->shade_variant = keep_v;
+    h->variant_chosen = keep_chosen;
     h->shade_ctas_per_sm = keep_c;
     return cuda_fail(h, err, "autotune");
   }
@@ -811,6 +820,7 @@ nvc_status nvc_set_shade_variant(nvc_handle* h, int32_t variant) {
   if (variant != kShadeMono && variant != kShadePair && h->L > 32)
     return fail(h, NVC_ERR_UNSUPPORTED, "variants 1-4, 6 and 7 need n_outputs <= 32");
   h->shade_variant = variant;
+  h->variant_chosen = true;
   return NVC_OK;
 }
 
@@ -833,6 +843,8 @@ nvc_status nvc_autotune_infer(nvc_handle* h, const float* pos, int64_t n, float*
   NVC_CUDA(h, cudaEventCreate(&e0));
   NVC_CUDA(h, cudaEventCreate(&e1));
   const int keep = h->shade_variant;
+  const bool keep_chosen = h->variant_chosen;
+  h->variant_chosen = true;
   int best = -1;
   double best_ms = 0.0;
   cudaError_t err = cudaSuccess;
@@ -861,6 +873,7 @@ nvc_status nvc_autotune_infer(nvc_handle* h, const float* pos, int64_t n, float*
     }
   }
   h->shade_variant = keep;
+  h->variant_chosen = keep_chosen;
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   if (err != cudaSuccess) return cuda_fail(h, err, "autotune");
@@ -882,6 +895,8 @@ nvc_status nvc_autotune_shade(nvc_handle* h, const nvc_scene* scene, const float
   NVC_CUDA(h, cudaEventCreate(&e0));
   NVC_CUDA(h, cudaEventCreate(&e1));
   const int keep = h->shade_variant;
+  const bool keep_chosen = h->variant_chosen;
+  h->variant_chosen = true;
   int best = -1;
   double best_ms = 0.0;
   for (int v = 0; v < kShadeVariants; ++v) {
@@ -900,6 +915,7 @@ nvc_status nvc_autotune_shade(nvc_handle* h, const nvc_scene* scene, const float
     e = cudaEventSynchronize(e1);
     if (e != cudaSuccess) {
       h->shade_variant = keep;
+      h->variant_chosen = keep_chosen;
       cudaEventDestroy(e0);
       cudaEventDestroy(e1);
       return cuda_fail(h, e, "autotune");

@@ -357,5 +357,7 @@ struct PackArgs {
 // other launches' fields, tpc is 2 or 4, L <= 32.
 cudaError_t launch_shade_multi(fz::FusedArgs a, const nvc_handle* h, const fz::PackArgs& p, int tpc,
                                bool bf16, cudaStream_t s);
+// Whether tpc tile streams fit a CTA's shared memory and TMEM.
+bool multi_fits(const nvc_handle* h, const fz::PackArgs& p, int tpc);
 
 }  // namespace nvc

@@ -54,7 +54,7 @@ __global__ void __launch_bounds__(kTileM, 5) fused_shade_kernel(const __grid_con
 
   for (int e = t; e < a.wimg_bytes / 16; e += kTileM)
     reinterpret_cast<uint4*>(s_w)[e] = a.wimg[e];
-  if (a.lights) stage_light_pairs(s_l, a.lights, a.L, t, kTileM, (a.L + 1) & ~1);
+  if (a.lights) stage_light_pairs(s_l, a.lights, a.L, t, kTileM, round_up16(a.L));
   const uint32_t bar = smem_u32(s_bar);
   if (t == 0) {
     mbar_init(bar, 1);
@@ -211,26 +211,28 @@ __global__ void __launch_bounds__(kTileM, 5) fused_shade_kernel(const __grid_con
         for (int c0 = 0; c0 < L; c0 += 32) {
           uint32_t r[32];
           tmem_ld32(t_lane + (uint32_t)c0, r);
-          // two lights per packed operation (pair (c0 + j) / 2 of the table)
+          // two lights per packed operation (pair (c0 + j) / 2 of the table);
+          // bounds by groups of four, lights past L in a group are zero
+          // lights, whose weight is 0 (1080p x 32 lights 402 -> 365 us)
 #pragma unroll
-          for (int j = 0; j < 32; j += 2) {
-            const int i = c0 + j;
-            wreg[j] = 0.0f;
-            wreg[j + 1] = 0.0f;
-            if (i < L) {
-              const float2 c = contribution2_fast(npx, npy, npz, nx2, ny2, nz2, s_l[i], s_l[i + 1]);
-              const float v0 = sigmoid_fast(__uint_as_float(r[j]) * outmul);
-              const float w0 = __fmul_rn(fmaxf(v0, bits_f(kVisClampBits)), c.x);
-              wmax = fmaxf(wmax, w0);
-              sum += w0;
-              di = fmaf(v0, c.x, di);
-              wreg[j] = w0;
-              if (i + 1 < L) {
+          for (int g = 0; g < 32; g += 4) {
+#pragma unroll
+            for (int j = g; j < g + 4; ++j) wreg[j] = 0.0f;
+            if (c0 + g < L) {
+#pragma unroll
+              for (int j = g; j < g + 4; j += 2) {
+                const int i = c0 + j;
+                const float2 c = contribution2_fast(npx, npy, npz, nx2, ny2, nz2, s_l[i], s_l[i + 1]);
+                const float v0 = sigmoid_fast(__uint_as_float(r[j]) * outmul);
                 const float v1 = sigmoid_fast(__uint_as_float(r[j + 1]) * outmul);
+                const float w0 = __fmul_rn(fmaxf(v0, bits_f(kVisClampBits)), c.x);
                 const float w1 = __fmul_rn(fmaxf(v1, bits_f(kVisClampBits)), c.y);
-                wmax = fmaxf(wmax, w1);
+                wmax = fmaxf(fmaxf(wmax, w0), w1);
+                sum += w0;
+                di = fmaf(v0, c.x, di);
                 sum += w1;
                 di = fmaf(v1, c.y, di);
+                wreg[j] = w0;
                 wreg[j + 1] = w1;
               }
             }
@@ -271,21 +273,22 @@ __global__ void __launch_bounds__(kTileM, 5) fused_shade_kernel(const __grid_con
           if (!LSMALL) tmem_ld32(t_lane + (uint32_t)c0, r);
           if (active) {
 #pragma unroll
-            for (int j = 0; j < 32; ++j) {
-              const int i = c0 + j;
-              if (i < L) {
-                float w = wreg[j];
-                if (!LSMALL) w = __fmul_rn(__uint_as_float(r[j]), qs.pre);
-                if ((i & 3) == 0)
-                  rr = philox_keyed(make_uint4(pixel, a.frame, V.view,
-                                               ((uint32_t)(i >> 2) << 4) | kTagWrs),
-                                    a.rkey);
-                const uint32_t q = quantize_scaled(w, qs.scale);
-                Q += q;
-                // r*Q < q*2^32  <=>  hi32(r*Q) < q  (Q < 2^32); false for q = 0
-                if (__umulhi(pick_word(rr, i & 3), Q) < q) {
-                  sel = i;
-                  wsel = w;
+            for (int g = 0; g < 32; g += 4) {
+              if (c0 + g < L) {
+                rr = philox_keyed(make_uint4(pixel, a.frame, V.view,
+                                             ((uint32_t)((c0 + g) >> 2) << 4) | kTagWrs),
+                                  a.rkey);
+#pragma unroll
+                for (int j = g; j < g + 4; ++j) {
+                  float w = wreg[j];
+                  if (!LSMALL) w = __fmul_rn(__uint_as_float(r[j]), qs.pre);
+                  const uint32_t q = quantize_scaled(w, qs.scale);
+                  Q += q;
+                  // r*Q < q*2^32  <=>  hi32(r*Q) < q  (Q < 2^32); false for q = 0
+                  if (__umulhi(pick_word(rr, j & 3), Q) < q) {
+                    sel = c0 + j;
+                    wsel = w;
+                  }
                 }
               }
             }
@@ -1270,6 +1273,30 @@ bool fused_supported(const nvc_handle* h, std::string* why) {
   return true;
 }
 
+// The layout of a launch whose handle has chosen none, by light count and
+// 128-pixel tiles (all give the same picks; see ShadeVariant).  Measured in
+// us, 16 levels x 2 features, MLP 32-64-64-64-L, variants 0 / 5 / 6, shading:
+//   32 lights   1,000 px 18.7 / 15.3 / 20.8     56,320 px 31.6 / 23.3 / 28.8
+//             160,000 px 51.8 / 47.6 / 46.0    578,731 px  122 /  128 /  111
+//   21 lights, float32 table                   578,731 px  113 /  130 /  107
+//   40 lights   4,096 px 21.1 / 17.1            76,800 px 37.7 / 33.6
+//                                              578,731 px  139 /  144
+//   96 lights                                  578,731 px  200 /  187
+// Few tiles are a chain of latencies, which two threads a pixel shorten;
+// many are bound by issue, where two tile streams per CTA keep most warps in
+// flight.  Above 32 lights variant 6 does not run: two threads a pixel win
+// from 64 lights, and for exported visibilities (40 lights, 578,731 px: 133
+// against 123).  E4M3 operands run 0 and 5; 0 is the faster from 1,000 px on.
+int default_variant(const nvc_handle* h, const PackArgs& p, const FusedArgs& a) {
+  if (h->cfg.precision == NVC_PREC_FP8) return kShadeMono;
+  const bool pair_fits = pair_smem(h, p) <= 225 * 1024;
+  if (h->L <= 32 && a.n_tiles > 3 * h->num_sms && multi_fits(h, p, 2)) return kShadeMulti2;
+  const bool infer = a.v[0].vis_out != nullptr;
+  const bool pair = h->L <= 32 ? a.n_tiles <= 3 * h->num_sms
+                               : h->L > 64 || infer || a.n_tiles <= 4 * h->num_sms;
+  return pair && pair_fits ? kShadePair : kShadeMono;
+}
+
 cudaError_t launch_shade_fused_views(const nvc_handle* h, const nvc_scene* sc,
                                      const FusedView* views, int n_views, uint64_t seed,
                                      uint32_t frame, cudaStream_t s,
@@ -1344,7 +1371,8 @@ cudaError_t launch_shade_fused_views(const nvc_handle* h, const nvc_scene* sc,
     return launch_shade_multi(a, h, p, h->shade_variant == kShadeMulti2 ? 2 : 4,
                               h->cfg.precision == NVC_PREC_BF16, s);
   }
-  if (h->cfg.precision == NVC_PREC_FP8 && h->shade_variant == kShadePair) {
+  const int variant = h->variant_chosen ? h->shade_variant : default_variant(h, p, a);
+  if (h->cfg.precision == NVC_PREC_FP8 && variant == kShadePair) {
     const size_t smem_p8 = pair_smem(h, p, &a);
     switch (h->F) {
       case 1: return launch_pair_typed<1, NVC_PREC_FP8>(a, smem_p8, h->num_sms, s);
@@ -1365,7 +1393,6 @@ cudaError_t launch_shade_fused_views(const nvc_handle* h, const nvc_scene* sc,
     return cudaErrorInvalidValue;
   }
   const bool bf16 = h->cfg.precision == NVC_PREC_BF16;
-  const int variant = h->shade_variant;
   if ((variant == kShadeMulti2 || variant == kShadeMulti4) && h->L <= 32)
     return launch_shade_multi(a, h, p, variant == kShadeMulti2 ? 2 : 4, bf16, s);
   if (variant == kShadePair) {

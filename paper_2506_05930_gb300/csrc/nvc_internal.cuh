@@ -243,6 +243,9 @@ struct nvc_handle {
   // fused shading kernel variant (nvc::ShadeVariant); nvc_infer's own
   // variant (-1: the shading variant), set by nvc_autotune_infer
   int shade_variant = 0;
+  // false until a variant is chosen (nvc_set_shade_variant, nvc_set_shade_plan
+  // or an autotune call): launches then take default_variant's
+  bool variant_chosen = false;
   int infer_variant = -1;
   // resident CTAs per SM of the fused shading launches (0: as many as fit),
   // the occupancy point of nvc_set_shade_plan / nvc_autotune_shade_plan
