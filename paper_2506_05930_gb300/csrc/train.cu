@@ -198,6 +198,13 @@ __device__ __forceinline__ bool nonzero4(float4 g) {
   return g.x != 0.0f || g.y != 0.0f || g.z != 0.0f || g.w != 0.0f;
 }
 
+// Whether every word of the gradient and both moments is +0.
+__device__ __forceinline__ bool untouched4(float4 g, float4 m, float4 v) {
+  return (__float_as_uint(g.x) | __float_as_uint(g.y) | __float_as_uint(g.z) | __float_as_uint(g.w) |
+          __float_as_uint(m.x) | __float_as_uint(m.y) | __float_as_uint(m.z) | __float_as_uint(m.w) |
+          __float_as_uint(v.x) | __float_as_uint(v.y) | __float_as_uint(v.z) | __float_as_uint(v.w)) == 0u;
+}
+
 // Element j (an MLP weight) of the 16-bit weight image, set to v.
 __device__ __forceinline__ void set_image(const MlpImageMap& mp, uint8_t* img, int64_t j, float v) {
   int k = 0;
@@ -263,6 +270,10 @@ __device__ __forceinline__ void adam_update(float* __restrict__ theta, float* __
     for (int u = 0; u < kAdamGroups; ++u) {
       const int64_t ee = e + u * stride;
       if (u > 0 && ee >= n4) break;
+      // rows no lattice corner hashes to (most of the coarse levels' tables)
+      // stay at zero moments: the update leaves them as they are, so nothing
+      // is stored (a quarter of the 1080p table; the frame 507 -> 498 us)
+      if (eps > 0.0f && untouched4(g[u], mm[u], vv[u])) continue;
       adam_scalar(th[u].x, g[u].x, mm[u].x, vv[u].x, sc, beta1, beta2, eps);
       adam_scalar(th[u].y, g[u].y, mm[u].y, vv[u].y, sc, beta1, beta2, eps);
       adam_scalar(th[u].z, g[u].z, mm[u].z, vv[u].z, sc, beta1, beta2, eps);
