@@ -18,8 +18,8 @@ namespace nvc {
 //   boxes, 24 bytes each: (lo_x, hi_x), (lo_y, hi_y), (lo_z, hi_z).
 // A slab's two planes go through each packed float32x2 subtraction and
 // multiplication (Blackwell's sub/mul.rn.f32x2), each lane the correctly
-// rounded operation of the scalar test; the sphere pairs are read with two
-// 16-byte loads and tested lane by lane in scalar operations.
+// rounded operation of the scalar test; the sphere pairs are held against the
+// segment two at a time (near_spheres), and tested exactly one by one.
 struct Occluders {
   const float4* sph;   // 2 float4 per sphere pair
   int n_pairs;
@@ -99,14 +99,6 @@ __device__ __forceinline__ bool sphere_lane_blocks(float px, float py, float pz,
   const float ey = __fsub_rn(cy, __fadd_rn(py, __fmul_rn(tc, dy)));
   const float ez = __fsub_rn(cz, __fadd_rn(pz, __fmul_rn(tc, dz)));
   return dot3_rn(ex, ey, ez, ex, ey, ez) < r2;
-}
-
-// Two spheres: A = {cx_a, cx_b, cy_a, cy_b}, B = {cz_a, cz_b, r_a^2, r_b^2}.
-__device__ __forceinline__ bool sphere_pair_blocks(float px, float py, float pz, float dx,
-                                                   float dy, float dz, float inv_dd, float4 A,
-                                                   float4 B) {
-  return sphere_lane_blocks(px, py, pz, dx, dy, dz, inv_dd, A.x, A.z, B.x, B.z) ||
-         sphere_lane_blocks(px, py, pz, dx, dy, dz, inv_dd, A.y, A.w, B.y, B.w);
 }
 
 // Closed slab test of one box when no component of d is zero: the entry and
@@ -203,18 +195,58 @@ __device__ __forceinline__ bool box_blocks(const Segment& g, const Occluders& oc
                             make_float2(g.iy, g.iy), make_float2(g.iz, g.iz), b);
 }
 
+// The spheres of pairs [k0, k1), at most 16 pairs, that may block the segment:
+// bit 2 (k - k0) + lane.  The exact test of a sphere is some 26 operations
+// that must stay scalar and unfused; this one, 13 packed ones a pair, asks
+// only whether the centre's distance from the segment's line clears the
+// radius by more than any rounding:
+//   oo - (o.d)^2 / dd > r^2,  o = c - x,
+// with oo scaled down by 2^-15, r^2 up by 2^-16 and 2^-15 (|x|^2 + |l|^2) added
+// to it (`slack`).  The exact test's error is a few 2^-24 of the coordinates
+// x, l, c, so of the squares at most 2^-18 (|x|^2 + |l|^2 + |c|^2 + r^2), and
+// |c|^2 <= 2 |x|^2 + 2 oo; this one's own is some 20 x 2^-24 of oo.  What is
+// not a number is kept.  (1080p temporal merge with its ray, 32 spheres + 32
+// boxes: 145 -> 127 us.)
+__device__ __forceinline__ uint32_t near_spheres(const Segment& g, const Occluders& occ, int k0, int k1,
+                                                 float slack) {
+  const float2 npx = make_float2(-g.px, -g.px), npy = make_float2(-g.py, -g.py),
+               npz = make_float2(-g.pz, -g.pz);
+  const float2 dx = make_float2(g.dx, g.dx), dy = make_float2(g.dy, g.dy), dz = make_float2(g.dz, g.dz);
+  const float2 ninv = make_float2(-g.inv_dd, -g.inv_dd);
+  uint32_t m = 0, bit = 1;
+#pragma unroll 4
+  for (int k = k0; k < k1; ++k, bit <<= 2) {
+    const float4 A = occ.sph[2 * k], B = occ.sph[2 * k + 1];
+    const float2 ox = __fadd2_rn(make_float2(A.x, A.y), npx);
+    const float2 oy = __fadd2_rn(make_float2(A.z, A.w), npy);
+    const float2 oz = __fadd2_rn(make_float2(B.x, B.y), npz);
+    const float2 od = __ffma2_rn(ox, dx, __ffma2_rn(oy, dy, __fmul2_rn(oz, dz)));
+    const float2 oo = __ffma2_rn(ox, ox, __ffma2_rn(oy, oy, __fmul2_rn(oz, oz)));
+    const float2 c = __ffma2_rn(
+        __fmul2_rn(od, ninv), od,
+        __ffma2_rn(oo, make_float2(1.0f - 0x1p-15f, 1.0f - 0x1p-15f),
+                   __fmul2_rn(make_float2(B.z, B.w), make_float2(-1.0f - 0x1p-16f, -1.0f - 0x1p-16f))));
+    if (!(c.x > slack)) m |= bit;
+    if (!(c.y > slack)) m |= bit << 1;
+  }
+  return m;
+}
+
 // Whether the segment from (px, py, pz) to the light at (lx, ly, lz) is
-// blocked by one of the staged occluders.
+// blocked by one of the staged occluders.  The spheres that near_spheres
+// keeps are tested exactly, then the boxes.
 __device__ __forceinline__ bool segment_blocked(float px, float py, float pz, float lx, float ly,
                                                 float lz, const Occluders& occ) {
   const Segment g = make_segment(px, py, pz, lx, ly, lz);
-  const float2 px2 = make_float2(px, px), py2 = make_float2(py, py), pz2 = make_float2(pz, pz);
+  const float slack = 0x1p-15f * (px * px + py * py + pz * pz + lx * lx + ly * ly + lz * lz);
   bool blocked = false;
-  for (int k = 0; k < occ.n_pairs && !blocked; ++k)
-    blocked = sphere_pair_blocks(px, py, pz, g.dx, g.dy, g.dz, g.inv_dd, occ.sph[2 * k],
-                                 occ.sph[2 * k + 1]);
-  if (blocked) return true;
+  for (int k0 = 0; k0 < occ.n_pairs; k0 += 16) {
+    uint32_t m = near_spheres(g, occ, k0, min(k0 + 16, occ.n_pairs), slack);
+    for (; m && !blocked; m &= m - 1) blocked = sphere_blocks(g, occ, 2 * k0 + __ffs(m) - 1);
+    if (blocked) return true;
+  }
   if (g.oblique) {
+    const float2 px2 = make_float2(px, px), py2 = make_float2(py, py), pz2 = make_float2(pz, pz);
     const float2 ix2 = make_float2(g.ix, g.ix), iy2 = make_float2(g.iy, g.iy),
                  iz2 = make_float2(g.iz, g.iz);
     for (int k = 0; k < occ.n_box && !blocked; ++k)
