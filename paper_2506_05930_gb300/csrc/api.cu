@@ -1119,10 +1119,10 @@ static nvc_status train_checks(nvc_handle* h, const nvc_scene* scene, const floa
 static nvc_status train_step_impl(nvc_handle* h, const nvc_scene* scene, const float* screen_pos,
                                   int64_t n_screen, uint64_t seed, uint32_t frame,
                                   double* loss_out, cudaStream_t s,
-                                  const nvc_clusters* clusters = nullptr) {
+                                  const nvc_clusters* clusters = nullptr, int frames = 0) {
   NVC_TRY(train_forward_backward(h, scene, screen_pos, n_screen, seed, frame, s, clusters));
   StageScope sc(h, s, 2);
-  NVC_CUDA(h, launch_adam(h, loss_out, true, s));
+  NVC_CUDA(h, launch_adam(h, loss_out, true, s, frames));
   // the Adam kernel rewrites a 16-bit weight image itself; E4M3 repacks
   MlpImageMap mp;
   const bool in_adam = mlp_image_map(h, &mp);
@@ -1323,7 +1323,7 @@ static nvc_status frame_body(nvc_handle* h, const nvc_scene* scene, const nvc_vi
   if (train_view != NVC_FRAME_NO_TRAINING) {
     const nvc_view* tv = train_view >= 0 ? &views[train_view] : nullptr;
     NVC_TRY(train_step_impl(h, scene, tv ? tv->pos : nullptr, tv ? tv->n_pixels : 0, seed,
-                            frame, loss_out, s));
+                            frame, loss_out, s, nullptr, 1));
   }
   const bool fused = h->cfg.precision != NVC_PREC_FP32;
   if (fused) {
@@ -1348,9 +1348,11 @@ static nvc_status frame_body(nvc_handle* h, const nvc_scene* scene, const nvc_vi
                          vw.idx, vw.pdf, vw.wsum, vw.radiance, 0, s));
     }
   }
-  bump_frames_kernel<<<1, 1, 0, s>>>(h->status);
-  NVC_CUDA(h, cudaGetLastError());
-  count_launches(h, 1);
+  if (train_view == NVC_FRAME_NO_TRAINING) {   // else the Adam step counted it
+    bump_frames_kernel<<<1, 1, 0, s>>>(h->status);
+    NVC_CUDA(h, cudaGetLastError());
+    count_launches(h, 1);
+  }
   return NVC_OK;
 }
 

@@ -46,21 +46,32 @@ inline Net make_net(const nvc_handle* h) {
   return n;
 }
 
-// Stages every layer transposed at sw; threads t of nt share the work, the
-// caller synchronises.  Reads run along the parameters' rows.
+// Stages every layer transposed at sw and, with `rows`, also as stored, [out]
+// [in rounded up to 8], at sw + r_off[k] (zero padding); threads t of nt share
+// the work, the caller synchronises.  Reads run along the parameters' rows.
+template <bool ROWS = false>
 __device__ __forceinline__ void stage_weights(const Net& net, const float* __restrict__ params,
-                                              float* sw, int t, int nt) {
+                                              float* sw, int t, int nt,
+                                              const int* r_off = nullptr) {
   for (int k = 0; k < net.n_layers; ++k) {
-    const int in = net.in[k], out = net.out[k], ld = net.po[k] + 4;
+    const int in = net.in[k], out = net.out[k], ld = net.po[k] + 4, pi = round8(in);
     const float* src = params + net.w_off[k];
     float* dst = sw + net.t_off[k];
-#pragma unroll 4
+    // j = e / in by a multiplication, exact for e < 2^16 and 2 <= in <= 128
+    const uint32_t inv = (uint32_t)(((1ull << 32) + in - 1) / in);
+#pragma unroll 8
     for (int e = t; e < in * out; e += nt) {
-      const int j = e / in, i = e - j * in;
-      dst[i * ld + j] = __ldg(src + e);
+      const int j = in == 1 ? e : (int)__umulhi((uint32_t)e, inv), i = e - j * in;
+      const float w = __ldg(src + e);
+      dst[i * ld + j] = w;
+      if constexpr (ROWS) sw[r_off[k] + j * pi + i] = w;
     }
     const int pad = net.po[k] - out;
     for (int e = t; e < in * pad; e += nt) dst[(e / pad) * ld + out + e % pad] = 0.0f;
+    if constexpr (ROWS) {
+      const int rp = pi - in;
+      for (int e = t; e < out * rp; e += nt) sw[r_off[k] + (e / rp) * pi + in + e % rp] = 0.0f;
+    }
   }
 }
 

@@ -103,17 +103,7 @@ __global__ void __launch_bounds__(kThreads) train_f32_kernel(const __grid_consta
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
   const int rg = lane & 7, og = lane >> 3;
   const int last = a.net.n_layers - 1, L = a.net.out[last];
-  stage_weights(a.net, a.params, sm, t, kThreads);
-  for (int k = 0; k <= last; ++k) {
-    const int in = a.net.in[k], out = a.net.out[k], pi = a.pi[k];
-    const float* src = a.params + a.net.w_off[k];
-    float* dst = sm + a.r_off[k];
-#pragma unroll 4
-    for (int e = t; e < out * pi; e += kThreads) {
-      const int j = e / pi, i = e - j * pi;
-      dst[e] = i < in ? __ldg(src + j * in + i) : 0.0f;
-    }
-  }
+  stage_weights<true>(a.net, a.params, sm, t, kThreads, a.r_off);
   double loss_acc = 0.0;
   bool bad = false;
   const int64_t n_tiles = (a.n + kRows - 1) / kRows;

@@ -336,7 +336,8 @@ cudaError_t launch_training_positions(const nvc_scene* sc, const float* screen_p
 cudaError_t launch_trace_visibility(const nvc_scene* sc, const float* pos, int64_t n,
                                     float* vis, cudaStream_t s);
 cudaError_t launch_loss_grad(nvc_handle* h, int64_t n, cudaStream_t s);
-cudaError_t launch_adam(nvc_handle* h, double* loss_out, bool apply, cudaStream_t s);
+// frames: added to the frame counter when the step is committed.
+cudaError_t launch_adam(nvc_handle* h, double* loss_out, bool apply, cudaStream_t s, int frames = 0);
 // Resident CTAs per SM of the Adam update (256 threads), for a one-wave grid.
 cudaError_t adam_occupancy(int* ctas_per_sm);
 cudaError_t launch_finish_gradient(nvc_handle* h, float* grad_out, double* loss_out,

@@ -156,8 +156,9 @@ __device__ __forceinline__ StepPlan plan_step(const StepArgs& a, const int32_t* 
 // The step's bookkeeping, once: the loss, the non-finite flag cleared for
 // the next step, and either the step count or the skip count and flag.
 __device__ __forceinline__ void commit_step(const StepPlan& pl, bool apply, double inv_count,
-                                            double* loss_out, int32_t* status) {
+                                            double* loss_out, int32_t* status, int frames = 0) {
   if (loss_out) *loss_out = pl.loss_sum * inv_count;
+  status[kStFrames] += frames;
   status[kStNonFinite] = 0;
   if (!apply) return;
   if (pl.nonfinite) {
@@ -308,6 +309,8 @@ __device__ __forceinline__ void adam_update(float* __restrict__ theta, float* __
 // parameters (the hash table), rewritten from the updated values.  img (may
 // be NULL): the tensor cores' 16-bit weight image, whose MLP weights are
 // rewritten from the updated values (the separate packing pass's job).
+// frames: added to the frame counter (1 for the step of a frame, which then
+// needs no launch of its own to count it: 2.8 of a small frame's 47 us).
 __global__ void __launch_bounds__(256) adam_kernel(float* __restrict__ theta,
                                                    float* __restrict__ grad,
                                                    float* __restrict__ m, float* __restrict__ v,
@@ -316,7 +319,8 @@ __global__ void __launch_bounds__(256) adam_kernel(float* __restrict__ theta,
                                                    StepArgs step, double inv_count,
                                                    double* loss_out, int32_t* status,
                                                    uint2* __restrict__ table16, int64_t n_table4,
-                                                   MlpImageMap mp, uint8_t* __restrict__ img) {
+                                                   MlpImageMap mp, uint8_t* __restrict__ img,
+                                                   int frames) {
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   float4* g4 = reinterpret_cast<float4*>(grad);
@@ -349,7 +353,7 @@ __global__ void __launch_bounds__(256) adam_kernel(float* __restrict__ theta,
     __threadfence();
     uint32_t* done = reinterpret_cast<uint32_t*>(status + kStAdamDone);
     if (atomicAdd(done, 1u) == gridDim.x - 1) {
-      commit_step(s_plan, true, inv_count, loss_out, status);
+      commit_step(s_plan, true, inv_count, loss_out, status, frames);
       atomicExch(done, 0u);
     }
   }
@@ -432,7 +436,7 @@ cudaError_t launch_loss_grad(nvc_handle* h, int64_t n, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-cudaError_t launch_adam(nvc_handle* h, double* loss_out, bool apply, cudaStream_t s) {
+cudaError_t launch_adam(nvc_handle* h, double* loss_out, bool apply, cudaStream_t s, int frames) {
   const nvc_config& c = h->cfg;
   const double inv_count = 1.0 / ((double)h->B * (double)h->L);
   StepArgs a{};
@@ -465,7 +469,8 @@ cudaError_t launch_adam(nvc_handle* h, double* loss_out, bool apply, cudaStream_
   uint8_t* img = mlp_image_map(h, &mp) ? static_cast<uint8_t*>(h->mlp_packed) : nullptr;
   adam_kernel<<<blocks, 256, 0, s>>>(h->params, h->grad, h->adam_m, h->adam_v, n4, h->n_params,
                                      c.beta1, c.beta2, c.eps, a, inv_count, loss_out, h->status,
-                                     reinterpret_cast<uint2*>(h->table16), h->n_table / 4, mp, img);
+                                     reinterpret_cast<uint2*>(h->table16), h->n_table / 4, mp, img,
+                                     frames);
   return cudaGetLastError();
 }
 
