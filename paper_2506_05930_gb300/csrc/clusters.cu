@@ -436,7 +436,7 @@ __global__ void __launch_bounds__(256) temporal_merge_kernel(
     int32_t* __restrict__ light_out, float* __restrict__ W_out, int32_t* __restrict__ M_out,
     float* __restrict__ estimate) {
   extern __shared__ float4 s_occ[];
-  Occluders occ = staged_occluders(s_occ, 0, 0);
+  Occluders occ = no_occluders(s_occ);
   if (estimate) {
     occ = stage_occluders(spheres, n_sph, boxes, n_box, s_occ, threadIdx.x, blockDim.x);
     __syncthreads();
@@ -508,6 +508,8 @@ cudaError_t launch_cluster_targets(const nvc_scene* sc, const nvc_clusters* cl, 
   if (n == 0) return cudaSuccess;
   const int64_t total = n * cl->k;
   const size_t smem = occluder_bytes(sc->n_spheres, sc->n_boxes);
+  const cudaError_t e = allow_smem(cluster_targets_kernel, smem);
+  if (e != cudaSuccess) return e;
   cluster_targets_kernel<<<(unsigned)((total + 255) / 256), 256, smem, s>>>(
       sc->lights, sc->spheres, sc->n_spheres, sc->boxes, sc->n_boxes, cl->offsets, cl->members,
       cl->k, pos, n, (uint32_t)seed, (uint32_t)(seed >> 32), frame, target);

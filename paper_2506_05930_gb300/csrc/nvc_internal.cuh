@@ -288,6 +288,13 @@ nvc_status validate_config(const nvc_config* c, std::string* why);
 // footprint and the device's per-SM limits.
 int blocks_per_sm(const void* func, int block, size_t dyn_smem);
 
+// Lets `kern` take `smem` bytes of dynamic shared memory (needed past 48 KB).
+template <typename K>
+cudaError_t allow_smem(K kern, size_t smem) {
+  return smem <= 48 * 1024 ? cudaSuccess
+                           : cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+}
+
 // ---- launchers (each returns cudaGetLastError() of its launches) ----------
 // encode.cu
 cudaError_t launch_encode_fwd(const nvc_handle* h, const float* pos, int64_t n, float* feat,

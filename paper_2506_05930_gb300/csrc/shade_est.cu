@@ -156,6 +156,8 @@ cudaError_t launch_shade_estimate(const nvc_scene* sc, const float* pos, const f
                                   cudaStream_t s) {
   if (n == 0) return cudaSuccess;
   const size_t smem = occluder_bytes(sc->n_spheres, sc->n_boxes);
+  const cudaError_t e = allow_smem(shade_estimate_kernel, smem);
+  if (e != cudaSuccess) return e;
   shade_estimate_kernel<<<grid_for(n, num_sms), 256, smem, s>>>(
       sc->lights, sc->spheres, sc->n_spheres, sc->boxes, sc->n_boxes, pos, nrm, n, idx, pdf,
       estimate, accum, count);

@@ -15,20 +15,22 @@ namespace nvc {
 //   sphere pairs, 32 bytes each: float4 {cx_a, cx_b, cy_a, cy_b}, float4
 //   {cz_a, cz_b, r_a^2, r_b^2} (r^2 = fl(r r)); an odd count's last slot is
 //   a sphere with r^2 = -1, which blocks nothing;
-//   boxes, 24 bytes each: (lo_x, hi_x), (lo_y, hi_y), (lo_z, hi_z).
-// A slab's two planes go through each packed float32x2 subtraction and
-// multiplication (Blackwell's sub/mul.rn.f32x2), each lane the correctly
-// rounded operation of the scalar test; the sphere pairs are held against the
-// segment two at a time (near_spheres), and tested exactly one by one.
+//   box pairs, 48 bytes each: per axis float4 {c_a, c_b, h_a, h_b}, centre and
+//   half extent, the latter rounded up by 2^-16 of the box's coordinates: for
+//   the tests that only drop boxes (near_boxes, hull_meets_box).  The exact
+//   slab test reads the box itself from the scene's array.
+// The pairs are held against a segment two occluders at a time (near_spheres,
+// near_boxes), and what stands is tested exactly one by one.
 struct Occluders {
   const float4* sph;   // 2 float4 per sphere pair
   int n_pairs;
-  const float2* box;   // 3 float2 per box
+  const float4* box;   // 3 float4 per box pair
   int n_box;
+  const float* boxes;  // the scene's boxes, lo and hi (global memory)
 };
 
 __host__ __device__ __forceinline__ size_t occluder_bytes(int n_sph, int n_box) {
-  return 32 * (size_t)((n_sph + 1) / 2) + 24 * (size_t)n_box;
+  return 32 * (size_t)((n_sph + 1) / 2) + 48 * (size_t)((n_box + 1) / 2);
 }
 
 // Stages the occluders at dst (16-byte aligned; occluder_bytes(...) long),
@@ -54,26 +56,31 @@ __device__ __forceinline__ Occluders stage_occluders(const float* __restrict__ s
     q[6] = sp.w;
   }
   float* b = f + 8 * o.n_pairs;
-  for (int e = tid; e < n_box; e += nthreads) {
-    const float* src = boxes + 6 * e;
+  for (int e = tid; e < ((n_box + 1) & ~1); e += nthreads) {
+    float* q = b + 12 * (e >> 1) + (e & 1);
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-      b[6 * e + 2 * a] = src[a];
-      b[6 * e + 2 * a + 1] = src[3 + a];
+      float lo = 0.0f, hi = 0.0f;   // an odd count's last slot: never read as a box
+      if (e < n_box) {
+        lo = boxes[6 * e + a];
+        hi = boxes[6 * e + 3 + a];
+      }
+      q[4 * a] = 0.5f * lo + 0.5f * hi;
+      q[4 * a + 2] = fabsf(0.5f * hi - 0.5f * lo) + 0x1p-16f * (fabsf(lo) + fabsf(hi));
     }
   }
-  o.box = reinterpret_cast<const float2*>(b);
+  o.box = reinterpret_cast<const float4*>(b);
   o.n_box = n_box;
+  o.boxes = boxes;
   return o;
 }
 
-// The view of occluders already staged at src (as stage_occluders left them).
-__device__ __forceinline__ Occluders staged_occluders(const void* src, int n_sph, int n_box) {
+// No occluders yet (kernels that stage them only when they need them).
+__device__ __forceinline__ Occluders no_occluders(const void* at) {
   Occluders o;
-  o.sph = reinterpret_cast<const float4*>(src);
-  o.n_pairs = (n_sph + 1) / 2;
-  o.box = reinterpret_cast<const float2*>(static_cast<const float*>(src) + 8 * o.n_pairs);
-  o.n_box = n_box;
+  o.sph = o.box = reinterpret_cast<const float4*>(at);
+  o.n_pairs = o.n_box = 0;
+  o.boxes = nullptr;
   return o;
 }
 
@@ -187,7 +194,9 @@ __device__ __forceinline__ bool sphere_blocks(const Segment& g, const Occluders&
 }
 
 __device__ __forceinline__ bool box_blocks(const Segment& g, const Occluders& occ, int i) {
-  const float2* b = occ.box + 3 * i;
+  const float* q = occ.boxes + 6 * i;
+  const float2 b[3] = {make_float2(__ldg(q), __ldg(q + 3)), make_float2(__ldg(q + 1), __ldg(q + 4)),
+                       make_float2(__ldg(q + 2), __ldg(q + 5))};
   if (!g.oblique)
     return box_blocks_general(g.px, g.py, g.pz, g.dx, g.dy, g.dz, g.ix, g.iy, g.iz, b);
   return box_blocks_oblique(make_float2(g.px, g.px), make_float2(g.py, g.py),
@@ -232,9 +241,49 @@ __device__ __forceinline__ uint32_t near_spheres(const Segment& g, const Occlude
   return m;
 }
 
+// The boxes of pairs [k0, k1), at most 16 pairs, that may block an oblique
+// segment: bit 2 (k - k0) + lane.  The slab test's two planes per axis are
+// (c -+ h - x) / d, so from centre and half extent near and far come without
+// a minimum and a maximum -- three packed operations an axis for two boxes --
+// and only the largest near and smallest far are left to the ALU, which the
+// exact test keeps busy with 13 operations a box.  A box is dropped when near
+// exceeds far by more than `slack`, 2^-16 of the coordinates of x and the
+// light times the largest |1 / d|: the exact test's planes and these ones are
+// off by some 4 x 2^-24 of (|x| + |c| + h) / |d|, the box's share of which is
+// in h.  What is not a number is kept.  (1080p frame 494 -> 489 us, temporal
+// merge with its ray 127 -> 114 us, each with 32 boxes.)
+__device__ __forceinline__ uint32_t near_boxes(const Segment& g, const Occluders& occ, int k0, int k1,
+                                               float slack) {
+  const float2 ix = make_float2(g.ix, g.ix), iy = make_float2(g.iy, g.iy), iz = make_float2(g.iz, g.iz);
+  const float2 ax = make_float2(fabsf(g.ix), fabsf(g.ix)), ay = make_float2(fabsf(g.iy), fabsf(g.iy)),
+               az = make_float2(fabsf(g.iz), fabsf(g.iz));
+  const float2 bx = make_float2(-ax.x, -ax.x), by = make_float2(-ay.x, -ay.x),
+               bz = make_float2(-az.x, -az.x);
+  const float sx = -g.px * g.ix, sy = -g.py * g.iy, sz = -g.pz * g.iz;
+  const float t0 = bits_f(kSegT0Bits), t1 = bits_f(kSegT1Bits);
+  uint32_t m = 0, bit = 1;
+#pragma unroll 4
+  for (int k = k0; k < k1; ++k, bit <<= 2) {
+    const float4 X = occ.box[3 * k], Y = occ.box[3 * k + 1], Z = occ.box[3 * k + 2];
+    const float2 hx = make_float2(X.z, X.w), hy = make_float2(Y.z, Y.w), hz = make_float2(Z.z, Z.w);
+    const float2 mx = __ffma2_rn(make_float2(X.x, X.y), ix, make_float2(sx, sx));
+    const float2 my = __ffma2_rn(make_float2(Y.x, Y.y), iy, make_float2(sy, sy));
+    const float2 mz = __ffma2_rn(make_float2(Z.x, Z.y), iz, make_float2(sz, sz));
+    const float2 nx = __ffma2_rn(hx, bx, mx), ny = __ffma2_rn(hy, by, my), nz = __ffma2_rn(hz, bz, mz);
+    const float2 fx = __ffma2_rn(hx, ax, mx), fy = __ffma2_rn(hy, ay, my), fz = __ffma2_rn(hz, az, mz);
+    const float na = fmaxf(fmaxf(fmaxf(nx.x, ny.x), nz.x), t0);
+    const float fa = fminf(fminf(fminf(fx.x, fy.x), fz.x), t1);
+    const float nb = fmaxf(fmaxf(fmaxf(nx.y, ny.y), nz.y), t0);
+    const float fb = fminf(fminf(fminf(fx.y, fy.y), fz.y), t1);
+    if (!(na - fa > slack)) m |= bit;
+    if (!(nb - fb > slack)) m |= bit << 1;
+  }
+  return 2 * k1 > occ.n_box ? m & ~(1u << (occ.n_box - 2 * k0)) : m;   // not the padding slot
+}
+
 // Whether the segment from (px, py, pz) to the light at (lx, ly, lz) is
-// blocked by one of the staged occluders.  The spheres that near_spheres
-// keeps are tested exactly, then the boxes.
+// blocked by one of the staged occluders: those that near_spheres and
+// near_boxes keep are tested exactly.
 __device__ __forceinline__ bool segment_blocked(float px, float py, float pz, float lx, float ly,
                                                 float lz, const Occluders& occ) {
   const Segment g = make_segment(px, py, pz, lx, ly, lz);
@@ -246,14 +295,18 @@ __device__ __forceinline__ bool segment_blocked(float px, float py, float pz, fl
     if (blocked) return true;
   }
   if (g.oblique) {
-    const float2 px2 = make_float2(px, px), py2 = make_float2(py, py), pz2 = make_float2(pz, pz);
-    const float2 ix2 = make_float2(g.ix, g.ix), iy2 = make_float2(g.iy, g.iy),
-                 iz2 = make_float2(g.iz, g.iz);
-    for (int k = 0; k < occ.n_box && !blocked; ++k)
-      blocked = box_blocks_oblique(px2, py2, pz2, ix2, iy2, iz2, occ.box + 3 * k);
+    const float far = 0x1p-16f *
+                      (fmaxf(fmaxf(fabsf(px), fabsf(py)), fabsf(pz)) +
+                       fmaxf(fmaxf(fabsf(lx), fabsf(ly)), fabsf(lz))) *
+                      fmaxf(fmaxf(fabsf(g.ix), fabsf(g.iy)), fabsf(g.iz));
+    const int n = (occ.n_box + 1) >> 1;
+    for (int k0 = 0; k0 < n; k0 += 16) {
+      uint32_t m = near_boxes(g, occ, k0, min(k0 + 16, n), far);
+      for (; m && !blocked; m &= m - 1) blocked = box_blocks(g, occ, 2 * k0 + __ffs(m) - 1);
+      if (blocked) return true;
+    }
   } else {
-    for (int k = 0; k < occ.n_box && !blocked; ++k)
-      blocked = box_blocks_general(px, py, pz, g.dx, g.dy, g.dz, g.ix, g.iy, g.iz, occ.box + 3 * k);
+    for (int k = 0; k < occ.n_box && !blocked; ++k) blocked = box_blocks(g, occ, k);
   }
   return blocked;
 }
@@ -334,18 +387,14 @@ __device__ __forceinline__ bool hull_meets_sphere(const WarpHull& w, const HullR
 
 __device__ __forceinline__ bool hull_meets_box(const WarpHull& w, const HullRay& r,
                                                const Occluders& occ, int i) {
-  const float2 bx = occ.box[3 * i], by = occ.box[3 * i + 1], bz = occ.box[3 * i + 2];
-  const float m = 0x1p-16f * (r.scale + fmaxf(fmaxf(fmaxf(fabsf(bx.x), fabsf(bx.y)),
-                                                   fmaxf(fabsf(by.x), fabsf(by.y))),
-                                             fmaxf(fabsf(bz.x), fabsf(bz.y))));
-  const float ax = (fminf(bx.x, bx.y) - w.hx - m - w.cx) * r.ix,
-              cx = (fmaxf(bx.x, bx.y) + w.hx + m - w.cx) * r.ix;
-  const float ay = (fminf(by.x, by.y) - w.hy - m - w.cy) * r.iy,
-              cy = (fmaxf(by.x, by.y) + w.hy + m - w.cy) * r.iy;
-  const float az = (fminf(bz.x, bz.y) - w.hz - m - w.cz) * r.iz,
-              cz = (fmaxf(bz.x, bz.y) + w.hz + m - w.cz) * r.iz;
-  const float tmin = fmaxf(fmaxf(fminf(ax, cx), fminf(ay, cy)), fmaxf(fminf(az, cz), 0.0f));
-  const float tmax = fminf(fminf(fmaxf(ax, cx), fmaxf(ay, cy)), fminf(fmaxf(az, cz), 1.0f));
+  const float* q = reinterpret_cast<const float*>(occ.box + 3 * (i >> 1)) + (i & 1);
+  const float m = 0x1p-16f * r.scale;   // the box's own share is in its half extents
+  const float ax = fabsf(r.ix), ay = fabsf(r.iy), az = fabsf(r.iz);
+  const float mx = (q[0] - w.cx) * r.ix, kx = (q[2] + w.hx + m) * ax;
+  const float my = (q[4] - w.cy) * r.iy, ky = (q[6] + w.hy + m) * ay;
+  const float mz = (q[8] - w.cz) * r.iz, kz = (q[10] + w.hz + m) * az;
+  const float tmin = fmaxf(fmaxf(mx - kx, my - ky), fmaxf(mz - kz, 0.0f));
+  const float tmax = fminf(fminf(mx + kx, my + ky), fminf(mz + kz, 1.0f));
   return !(tmin > tmax);
 }
 

@@ -407,6 +407,8 @@ cudaError_t launch_training_data(const nvc_scene* sc, const float* screen_pos, i
     return launch_training_positions(sc, screen_pos, n_screen, batch, seed, frame, pos, s, n_world);
   const int64_t total = batch * sc->n_lights;
   const size_t smem = occluder_bytes(sc->n_spheres, sc->n_boxes);
+  const cudaError_t e = allow_smem(trace_visibility_kernel<true>, smem);
+  if (e != cudaSuccess) return e;
   trace_visibility_kernel<true><<<(unsigned)((total + 255) / 256), 256, smem, s>>>(
       sc->lights, sc->n_lights, sc->spheres, sc->n_spheres, sc->boxes, sc->n_boxes, pos, batch,
       vis, pos_gen(sc, screen_pos, n_screen, batch, seed, frame, n_world));
@@ -418,6 +420,8 @@ cudaError_t launch_trace_visibility(const nvc_scene* sc, const float* pos, int64
   if (n == 0) return cudaSuccess;
   const int64_t total = n * sc->n_lights;
   const size_t smem = occluder_bytes(sc->n_spheres, sc->n_boxes);
+  const cudaError_t e = allow_smem(trace_visibility_kernel<false>, smem);
+  if (e != cudaSuccess) return e;
   trace_visibility_kernel<false><<<(unsigned)((total + 255) / 256), 256, smem, s>>>(
       sc->lights, sc->n_lights, sc->spheres, sc->n_spheres, sc->boxes, sc->n_boxes,
       const_cast<float*>(pos), n, vis, PosGen{});

@@ -161,7 +161,7 @@ __global__ void __launch_bounds__(kTileM * NG, 1) train_tc_kernel(const __grid_c
   __shared__ float s_pos[GEN ? 3 * kTileM : 1];
   float4* s_lt = reinterpret_cast<float4*>(smem + a.occ_off);
   uint8_t* s_tgt = smem + a.tgt_off;
-  Occluders occ = staged_occluders(s_lt + a.L, 0, 0);
+  Occluders occ = no_occluders(s_lt + a.L);
   if constexpr (GEN) {
     occ = stage_occluders(a.spheres, a.n_sph, a.boxes, a.n_box, s_lt + a.L, threadIdx.x, kThreads);
     for (int e = threadIdx.x; e < a.L; e += kThreads)
