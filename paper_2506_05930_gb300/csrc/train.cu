@@ -113,13 +113,11 @@ __device__ __forceinline__ double pow_int(double b, int t) {
   return r;
 }
 
-// The step's constants, read from the loss partials and the status words
-// (not changed here): loss = sum of partials (lane-strided over one warp,
-// then a shuffle tree) x inv_count; whether the step applies (all gradients
-// finite); step t, bias corrections and the scheduled learning rate.
+// The step's constants, read from the status words (not changed here):
+// whether the step applies (all gradients finite); step t, bias corrections
+// and the scheduled learning rate.
 struct StepPlan {
   AdamScalars sc;
-  double loss_sum;
   int t;
   bool nonfinite;
 };
@@ -135,10 +133,6 @@ struct StepArgs {
 // Called by all 32 lanes of one warp; lane 0's result is the plan.
 __device__ __forceinline__ StepPlan plan_step(const StepArgs& a, const int32_t* status) {
   StepPlan pl{};
-  double s = 0.0;
-  for (int i = threadIdx.x & 31; i < a.n_partials; i += 32) s += a.partials[i];
-  for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-  pl.loss_sum = s;
   pl.nonfinite = status[kStNonFinite] != 0;
   pl.t = status[kStStep] + 1;
   double lr = a.lr0;
@@ -146,18 +140,31 @@ __device__ __forceinline__ StepPlan plan_step(const StepArgs& a, const int32_t* 
     const int k = pl.t - 1 < a.ramp ? pl.t - 1 : a.ramp;
     lr = (double)a.lr0 + ((double)a.lr_end - (double)a.lr0) * (double)k / (double)a.ramp;
   }
-  pl.sc.lr_over_bc1 = (float)(lr / (1.0 - pow_int(a.beta1, pl.t)));
-  pl.sc.inv_bc2 = (float)(1.0 / (1.0 - pow_int(a.beta2, pl.t)));
+  // lr / (1 - b1^t) in the even lanes, 1 / (1 - b2^t) in the odd ones: one
+  // chain of double-precision work instead of two through the same pipe
+  const bool odd = threadIdx.x & 1;
+  const double bc = (odd ? 1.0 : lr) / (1.0 - pow_int(odd ? a.beta2 : a.beta1, pl.t));
+  pl.sc.lr_over_bc1 = (float)bc;
+  pl.sc.inv_bc2 = (float)__shfl_down_sync(0xffffffffu, bc, 1);
   pl.sc.inv_scale = a.inv_scale;
   pl.sc.skip = pl.nonfinite ? 1 : 0;
   return pl;
 }
 
-// The step's bookkeeping, once: the loss, the non-finite flag cleared for
-// the next step, and either the step count or the skip count and flag.
-__device__ __forceinline__ void commit_step(const StepPlan& pl, bool apply, double inv_count,
-                                            double* loss_out, int32_t* status, int frames = 0) {
-  if (loss_out) *loss_out = pl.loss_sum * inv_count;
+// The step's loss: the sum of the partials (lane-strided over one warp, then a
+// shuffle tree) x inv_count.  The update does not wait for it: one warp of
+// one CTA forms it beside the planning warp.
+__device__ __forceinline__ void write_loss(const StepArgs& a, double inv_count, double* loss_out) {
+  double s = 0.0;
+  for (int i = threadIdx.x & 31; i < a.n_partials; i += 32) s += a.partials[i];
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+  if ((threadIdx.x & 31) == 0) *loss_out = s * inv_count;
+}
+
+// The step's bookkeeping, once: the non-finite flag cleared for the next
+// step, and either the step count or the skip count and flag.
+__device__ __forceinline__ void commit_step(const StepPlan& pl, bool apply, int32_t* status,
+                                            int frames = 0) {
   status[kStFrames] += frames;
   status[kStNonFinite] = 0;
   if (!apply) return;
@@ -174,7 +181,8 @@ __device__ __forceinline__ void commit_step(const StepPlan& pl, bool apply, doub
 __global__ void adam_prologue_kernel(StepArgs a, double inv_count, double* loss_out,
                                      int32_t* status) {
   const StepPlan pl = plan_step(a, status);
-  if (threadIdx.x == 0) commit_step(pl, false, inv_count, loss_out, status);
+  if (loss_out) write_loss(a, inv_count, loss_out);
+  if (threadIdx.x == 0) commit_step(pl, false, status);
 }
 
 // theta -= (lr / bc1) m / (sqrt(v / bc2) + eps), after m, v updates with the
@@ -337,6 +345,8 @@ __global__ void __launch_bounds__(256) adam_kernel(float* __restrict__ theta,
   if (threadIdx.x < 32) {
     const StepPlan pl = plan_step(step, status);
     if (threadIdx.x == 0) s_plan = pl;
+  } else if (threadIdx.x < 64 && blockIdx.x == 0 && loss_out) {
+    write_loss(step, inv_count, loss_out);
   }
   __syncthreads();
   const AdamScalars sc = s_plan.sc;
@@ -353,7 +363,7 @@ __global__ void __launch_bounds__(256) adam_kernel(float* __restrict__ theta,
     __threadfence();
     uint32_t* done = reinterpret_cast<uint32_t*>(status + kStAdamDone);
     if (atomicAdd(done, 1u) == gridDim.x - 1) {
-      commit_step(s_plan, true, inv_count, loss_out, status, frames);
+      commit_step(s_plan, true, status, frames);
       atomicExch(done, 0u);
     }
   }
