@@ -175,10 +175,11 @@ nvc_status nvc_set_table_precision(nvc_handle* h, int32_t precision, void* strea
 nvc_status nvc_get_state(nvc_handle* h, float* params, float* adam_m, float* adam_v,
                          void* stream);
 
-/* Capacity, in pixels, of the buffers the separate-kernel shading path
- * (nvc_shade with fused = 0, and FP32 nvc_infer) stages encoded features and
- * visibility in; larger inputs are processed in chunks of this size.  The
- * default is 65,536.  Synchronous; reallocates. */
+/* Capacity, in pixels, of the buffers that float32 nvc_sampler_weights, and
+ * nvc_shade with fused = 0 for networks whose outputs do not fit on chip
+ * beside their weights, stage encoded features and visibility in; larger
+ * inputs are processed in chunks of this size.  The default is 65,536.
+ * Synchronous; reallocates. */
 nvc_status nvc_set_staging(nvc_handle* h, int64_t max_pixels);
 
 /* Synchronises `stream`, then reads the device status into *out (host). */
@@ -249,8 +250,8 @@ nvc_status nvc_direct_illum(nvc_handle* h, const nvc_scene* scene, const float* 
 /* The per-pixel hot path in one pass: inference, WRS and Neural DI.
  * Outputs (device [n], any may be NULL) as nvc_wrs_sample and
  * nvc_direct_illum.  fused != 0 runs the single fused kernel of the
- * configuration's precision; fused == 0 runs the separate FP32 kernels
- * (encode, MLP, sampling) with visibility staged in the handle. */
+ * configuration's precision; fused == 0 runs the float32 kernel on the
+ * master parameters. */
 nvc_status nvc_shade(nvc_handle* h, const nvc_scene* scene, const float* pos,
                      const float* nrm, int64_t n, uint64_t seed, uint32_t frame,
                      uint32_t view, int64_t pixel_offset, int32_t* idx, float* pdf,

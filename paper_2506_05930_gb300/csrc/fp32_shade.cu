@@ -212,13 +212,90 @@ __global__ void __launch_bounds__(kWarps * 32, 3) shade_f32_kernel(const __grid_
   }
 }
 
+// Sampling and Neural DI on visibilities in memory (vis [n][L]), a pixel per
+// thread: the second half of the staged form below.
+__global__ void __launch_bounds__(128) shade_from_vis_kernel(
+    const float* __restrict__ lights, int L, const float* __restrict__ pos,
+    const float* __restrict__ nrm, const float* __restrict__ vis, int64_t n, uint32_t k0,
+    uint32_t k1, uint32_t frame, uint32_t view, int64_t pixel_offset, int32_t* __restrict__ idx,
+    float* __restrict__ pdf, float* __restrict__ wsum, float* __restrict__ radiance, float neg0) {
+  extern __shared__ float4 s_lights[];
+  bool lights_ok = true;
+  for (int e = threadIdx.x; e < ((L + 3) & ~3); e += blockDim.x) {
+    float4 l = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (e < L) l = reinterpret_cast<const float4*>(lights)[e];
+    l.w = __fmul_rn(l.w, bits_f(kInvPiBits));
+    xp::put_light(s_lights, e, l);
+    lights_ok = lights_ok && xp::light_ok(l);
+  }
+  lights_ok = __syncthreads_and(lights_ok) != 0;
+  const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (p >= n) return;
+  const float px = pos[3 * p], py = pos[3 * p + 1], pz = pos[3 * p + 2];
+  const xp::Pixel pp = xp::make_pixel(px, py, pz, nrm[3 * p], nrm[3 * p + 1], nrm[3 * p + 2], neg0,
+                                      lights_ok);
+  const float* vp = vis + p * L;
+  auto weights4 = [&](int i0, float (&c)[4], float (&v)[4], float (&w)[4]) {
+    xp::staged_contributions<2>(pp, s_lights + i0, c);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      v[q] = i0 + q < L ? __ldg(vp + i0 + q) : 0.0f;
+      w[q] = __fmul_rn(fmaxf(v[q], bits_f(kVisClampBits)), c[q]);
+    }
+  };
+  float wmax = 0.0f, sum = 0.0f, di = 0.0f;
+  for (int i0 = 0; i0 < L; i0 += 4) {
+    float c[4], v[4], w[4];
+    weights4(i0, c, v, w);
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      if (i0 + q < L) {
+        wmax = fmaxf(wmax, w[q]);
+        sum += w[q];
+        di = fmaf(v[q], c[q], di);
+      }
+  }
+  int sel = -1;
+  float wsel = 0.0f;
+  if (wmax > 0.0f) {
+    const bool finite = wmax <= FLT_MAX;   // else quantize_weight itself
+    const fz::QuantScale qs = fz::quant_scale(wmax);
+    const int e = ilogbf(wmax);
+    const uint32_t pixel = (uint32_t)(pixel_offset + p);
+    uint64_t Q = 0;
+    for (int i0 = 0; i0 < L; i0 += 4) {
+      float c[4], v[4], w[4];
+      weights4(i0, c, v, w);
+      const uint4 r = philox4x32_10(
+          make_uint4(pixel, frame, view, ((uint32_t)(i0 >> 2) << 4) | kTagWrs), k0, k1);
+#pragma unroll
+      for (int q4 = 0; q4 < 4; ++q4) {
+        if (i0 + q4 < L) {
+          const uint32_t q = finite ? fz::quantize_scaled(__fmul_rn(w[q4], qs.pre), qs.scale)
+                                    : quantize_weight(w[q4], e);
+          Q += q;
+          if (q != 0u && (uint64_t)fz::pick_word(r, q4) * Q < ((uint64_t)q << 32)) {
+            sel = i0 + q4;
+            wsel = w[q4];
+          }
+        }
+      }
+    }
+  }
+  if (idx) idx[p] = sel;
+  if (pdf) pdf[p] = sel >= 0 ? wsel / sum : 0.0f;
+  if (wsum) wsum[p] = sum;
+  if (radiance) radiance[p] = di;
+}
+
 // Shared memory with `warps` warps per CTA; fills the plan when `a` is given.
-size_t plan_smem(const nvc_handle* h, const Net& net, int warps, ShadeArgs* a) {
+// shade: the outputs stay in shared memory too.
+size_t plan_smem(const nvc_handle* h, const Net& net, int warps, bool shade, ShadeArgs* a) {
   // activation k (0: the encoded input, n_layers: the outputs) lies in area
   // k & 1; one area serves both while every layer is one 32-output pass,
   // whose products are all read before the first is written back
   int dims[2] = {h->din, 0}, widest = 0;
-  for (int k = 0; k < net.n_layers; ++k) {
+  for (int k = 0; k < net.n_layers - (shade ? 0 : 1); ++k) {
     int& d = dims[(k + 1) & 1];
     d = net.po[k] > d ? net.po[k] : d;
     widest = net.po[k] > widest ? net.po[k] : widest;
@@ -243,8 +320,8 @@ cudaError_t launch_typed(ShadeArgs& a, const nvc_handle* h, cudaStream_t s) {
   // warps on every SM would take, else eight
   const int64_t tiles = (a.n + kRows - 1) / kRows;
   int warps = tiles >= (int64_t)kWarps * h->num_sms ? kWarps : 4;
-  size_t smem = plan_smem(h, a.net, warps, &a);
-  while (smem > 227 * 1024 && warps > 1) smem = plan_smem(h, a.net, warps /= 2, &a);
+  size_t smem = plan_smem(h, a.net, warps, SHADE, &a);
+  while (smem > 227 * 1024 && warps > 1) smem = plan_smem(h, a.net, warps /= 2, SHADE, &a);
   if (smem > 227 * 1024) return cudaErrorInvalidConfiguration;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
@@ -304,7 +381,25 @@ cudaError_t launch_shade_f32(const nvc_handle* h, const nvc_scene* sc, const flo
   a.pdf = pdf;
   a.wsum = wsum;
   a.radiance = radiance;
-  return launch<true>(a, h, s);
+  // While four warps' activations, outputs among them, fit beside the weights,
+  // all on chip; a wider output layer leaves room for fewer warps than the SM
+  // has schedulers, and its visibilities go through the handle's staging.
+  // MLP 32-64-64-64-L, 578,731 pixels, on chip / staged (and the three-kernel
+  // form before) in us: 32 lights 476 / 769 (1,395), 128 1,434 / 1,533
+  // (2,999), 192 3,783 / 2,598 (4,094), 256 4,733 / 3,210 (4,771).
+  if (plan_smem(h, a.net, 4, true, nullptr) <= 227 * 1024) return launch<true>(a, h, s);
+  const size_t smem = sizeof(float4) * ((h->L + 3) & ~3);
+  for (int64_t o = 0; o < n; o += h->stage_pixels) {
+    const int64_t m = n - o < h->stage_pixels ? n - o : h->stage_pixels;
+    cudaError_t e = launch_infer_f32(h, pos + 3 * o, m, h->s_vis, s);
+    if (e != cudaSuccess) return e;
+    shade_from_vis_kernel<<<(unsigned)((m + 127) / 128), 128, smem, s>>>(
+        sc->lights, h->L, pos + 3 * o, nrm + 3 * o, h->s_vis, m, a.k0, a.k1, frame, view,
+        pixel_offset + o, idx ? idx + o : nullptr, pdf ? pdf + o : nullptr,
+        wsum ? wsum + o : nullptr, radiance ? radiance + o : nullptr, a.neg0);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
 }  // namespace nvc

@@ -50,6 +50,7 @@ def test_inference_and_shading_equal_the_separate_kernels(F, levels, hidden, L, 
     odd = torch.full((n * L + 1,), -1.0, device="cuda")[1:].view(n, L)   # 4-byte aligned rows
     nvc.nvc_infer(cache.handle, pos, odd)
     assert torch.equal(odd, ref)
+    nvc.nvc_set_staging(cache.handle, 1024)     # the widest networks go through it in chunks
     out = cache.shade(scene, pos, nrm, seed=(3 << 32) + 9, frame=7, view=2, pixel_offset=11, fused=False)
     c, w = torch.empty((n, L), device="cuda"), torch.empty((n, L), device="cuda")
     nvc.nvc_light_weights(scene, pos, nrm, ref, c, w)
