@@ -251,9 +251,9 @@ def clustered_alu_ops(n_lights, k, n_pixels):
 # Per-launch DRAM traffic of the dominant kernel from the ncu capture named in
 # profiles/ (None once the kernel has changed since that capture); the fused
 # shading kernel's by variant (the 1080p frame's launch).
-KERNEL_TRAFFIC = {"fused_shade": {6: 78.75e6, 7: 83.04e6}, "adam": 460.4e6,
+KERNEL_TRAFFIC = {"fused_shade": {6: 78.75e6, 7: 83.04e6}, "adam": None,
                   # 1080p launch with the shadow ray (light, W and estimate written)
-                  "sample_clustered": 336.78e6}
+                  "sample_clustered": 337.34e6}
 
 
 # ------------------------------------------------------------- our arm ----
@@ -686,7 +686,7 @@ def measure_clustered(args, gb, stream):
             "sample_with_shadow_ray_ms": sample_vis_ms,
             f"sample_with_shadow_ray_ms_at_{PAPER_SCALE_LIGHTS}_lights": sample_vis_big_ms,
             "note": "first-step weights max(v, 0.001) alone (NVC_CLUSTER_WEIGHT_VISIBILITY)"},
-        "roofline": {"kernel": "sample_clustered_kernel (no shadow ray)", "bound": "alu",
+        "roofline": {"kernel": "sample_sum_kernel (no shadow ray)", "bound": "alu",
                      "achieved": ops / (sampler_ms * 1e-3) / 1e12, "peak": peak / 1e12,
                      "unit": "Tops/s", "frac": ops / (sampler_ms * 1e-3) / peak,
                      "ops_per_pixel": ops / P,
@@ -918,7 +918,9 @@ def run_ours(args):
     adam_view = {"kernel": "adam", "bound": "hbm",
                  "achieved": alg["adam_bytes"] / adam_s / 1e9 if adam_s > 0 else None,
                  "peak": pk["hbm"], "unit": "GB/s", "peak_source": pk["src"] + " (MEASURED_PEAKS hbm_gbs)",
-                 "traffic": KERNEL_TRAFFIC["adam"]}
+                 "traffic": KERNEL_TRAFFIC["adam"],
+                 "note": "achieved counts every row as written; rows that never had a gradient "
+                         "are read and left alone"}
     tensor_view = {"kernel": "fused_shade MLP share", "bound": "tensor",
                    "achieved": alg["shade_flops"] / shade_s / 1e12, "peak": pk["bf16_sustained"],
                    "unit": "TFLOP/s", "peak_source": pk["src"] + " bf16 sustained (fp16 same rate)"}
