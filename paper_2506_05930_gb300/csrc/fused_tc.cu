@@ -212,8 +212,10 @@ __global__ void __launch_bounds__(kTileM, 5) fused_shade_kernel(const __grid_con
           uint32_t r[32];
           tmem_ld32(t_lane + (uint32_t)c0, r);
           // two lights per packed operation (pair (c0 + j) / 2 of the table);
-          // bounds by groups of four, lights past L in a group are zero
-          // lights, whose weight is 0 (1080p x 32 lights 402 -> 365 us)
+          // bounds by groups of four, lights past L in a group are zero lights
+          // with a cleared logit, whose terms are 0 (1080p x 32 lights 402 ->
+          // 365 us)
+          if ((L & 3) && L - c0 < 32) clear_past(r, L - c0);
 #pragma unroll
           for (int g = 0; g < 32; g += 4) {
 #pragma unroll
@@ -333,8 +335,8 @@ __global__ void __launch_bounds__(kTileM, 5) fused_shade_kernel(const __grid_con
 // the picks are the same integers from the same float32 weights.
 //
 // The light table is padded to whole 16-light chunks with zero lights, whose
-// weight is 0 whatever the padded logit says, so the sampler's loops carry no
-// bounds: with a bound per light the compiler kept a compare and a predicate
+// terms are 0 with the last chunk's padded logits cleared (clear_past), so the
+// sampler's loops carry no bounds: with a bound per light the compiler kept a compare and a predicate
 // on every operation.  3840x2160 x 256 lights, FP16: 6.87 -> 5.03 ms; four
 // views of 128 lights (14,976,000 random points): 7.97 -> 7.75 ms, there with
 // half the time in the encode's scattered row reads (load_x_pairs).  Four threads per pixel
@@ -536,6 +538,7 @@ __global__ void __launch_bounds__(2 * kTileM, MINB) fused_shade_pair_kernel(cons
         for (int c0 = lo; c0 < hi; c0 += 16) {
           uint32_t r[16];
           tmem_ld16(t_lane + (uint32_t)c0, r);
+          if (L - c0 < 16) clear_past(r, L - c0);
           // two lights per packed operation (pair (c0 + j) / 2 of the table)
 #pragma unroll
           for (int j = 0; j < 16; j += 2) {
