@@ -291,7 +291,10 @@ nvc_status nvc_calibrate(nvc_handle* h, const float* pos, int64_t n, void* strea
  * outputs, 5 sums w and the Neural DI terms over lights [0, H) and [H, L)
  * separately (H = ceil(ceil(L / 2) / 16) * 16), which can change the last
  * bits of wsum, pdf and radiance.  A handle on which none was chosen (by the
- * calls below) takes 0, 5 or 6 by its light and pixel count. */
+ * calls below) takes 0, 5 or 6 by its light count, and by the pixel count
+ * only among those that sum alike there, so that a pixel's outputs are the
+ * same in every launch: shards of an image and views of a frame equal the
+ * whole bit for bit. */
 #define NVC_SHADE_VARIANTS 8
 
 /* Chooses the fused-kernel variant that nvc_infer runs (the variants give

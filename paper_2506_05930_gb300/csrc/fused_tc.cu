@@ -1277,27 +1277,34 @@ bool fused_supported(const nvc_handle* h, std::string* why) {
 }
 
 // The layout of a launch whose handle has chosen none, by light count and
-// 128-pixel tiles (all give the same picks; see ShadeVariant).  Measured in
-// us, 16 levels x 2 features, MLP 32-64-64-64-L, variants 0 / 5 / 6, shading:
-//   32 lights   1,000 px 18.7 / 15.3 / 20.8     56,320 px 31.6 / 23.3 / 28.8
-//             160,000 px 51.8 / 47.6 / 46.0    578,731 px  122 /  128 /  111
+// 128-pixel tiles.  All give the same picks; variants 0 and 6 also give the
+// same sums, which variant 5 adds by halves (see ShadeVariant).  So that a
+// pixel's outputs do not depend on how many others share its launch, the tile
+// count only chooses between layouts with the same sums: 0 and 6, and 5 among
+// them where one half holds every light (up to 16) or nothing is summed
+// (exported visibilities).  Measured in us, 16 levels x 2 features, MLP
+// 32-64-64-64-L, variants 0 / 5 / 6, shading of a heightfield:
+//   32 lights   1,000 px 18.7 / 15.3 / 20.8      9,728 px 18.6 / 15.2 / 20.6
+//              20,000 px 23.4 / 18.5 / 20.6     56,320 px 29.4 / 22.6 / 26.3
+//             129,600 px 43.6 / 36.9 / 37.3    578,731 px  122 /  128 /  111
+//   17 lights   9,728 px 18.6 / 15.0 / 20.9     20,000 px 22.5 / 18.5 / 20.6
 //   21 lights, float32 table                   578,731 px  113 /  130 /  107
 //   40 lights   4,096 px 21.1 / 17.1            76,800 px 37.7 / 33.6
 //                                              578,731 px  139 /  144
 //   96 lights                                  578,731 px  200 /  187
 // Few tiles are a chain of latencies, which two threads a pixel shorten;
 // many are bound by issue, where two tile streams per CTA keep most warps in
-// flight.  Above 32 lights variant 6 does not run: two threads a pixel win
-// from 64 lights, and for exported visibilities (40 lights, 578,731 px: 133
-// against 123).  E4M3 operands run 0 and 5; 0 is the faster from 1,000 px on.
+// flight, from about one tile per SM on.  Above 32 lights variant 6 does not
+// run: two threads a pixel win from 64 lights, and for exported visibilities
+// (40 lights, 578,731 px: 133 against 123).  E4M3 operands run 0 and 5; 0 is
+// the faster from 1,000 px on.
 int default_variant(const nvc_handle* h, const PackArgs& p, const FusedArgs& a) {
   if (h->cfg.precision == NVC_PREC_FP8) return kShadeMono;
-  const bool pair_fits = pair_smem(h, p) <= 225 * 1024;
-  if (h->L <= 32 && a.n_tiles > 3 * h->num_sms && multi_fits(h, p, 2)) return kShadeMulti2;
   const bool infer = a.v[0].vis_out != nullptr;
-  const bool pair = h->L <= 32 ? a.n_tiles <= 3 * h->num_sms
-                               : h->L > 64 || infer || a.n_tiles <= 4 * h->num_sms;
-  return pair && pair_fits ? kShadePair : kShadeMono;
+  const bool pair_fits = pair_smem(h, p) <= 225 * 1024;
+  if (h->L > 32) return (h->L > 64 || infer) && pair_fits ? kShadePair : kShadeMono;
+  if ((h->L <= 16 || infer) && a.n_tiles <= 3 * h->num_sms && pair_fits) return kShadePair;
+  return a.n_tiles > h->num_sms && multi_fits(h, p, 2) ? kShadeMulti2 : kShadeMono;
 }
 
 cudaError_t launch_shade_fused_views(const nvc_handle* h, const nvc_scene* sc,
