@@ -354,7 +354,11 @@ __device__ __forceinline__ void pair_sync(int warp) {
 
 // MINB: CTAs per SM its registers leave room for; two above 128 lights, where
 // TMEM takes no more (at three, 80 registers a thread, the sampler spills).
-template <int F, int PREC, bool HSMALL, int MINB>
+// VIS: the launch exports visibilities, and the sampler is left out of the
+// code; with it in, the encode's loop was scheduled 2 to 5% slower (1080p x 32
+// lights 361 -> 330 us, 1003x577 x 96 lights 180 -> 173, 1080p random points x
+// 128 lights 1,358 -> 1,324).
+template <int F, int PREC, bool HSMALL, int MINB, bool VIS = false>
 __global__ void __launch_bounds__(2 * kTileM, MINB) fused_shade_pair_kernel(const __grid_constant__ FusedArgs a) {
   constexpr int kThreads = 2 * kTileM;
   extern __shared__ __align__(1024) uint8_t smem[];
@@ -441,7 +445,11 @@ __global__ void __launch_bounds__(2 * kTileM, MINB) fused_shade_pair_kernel(cons
               pack_chunk<PREC, CH>(fv, s_in0);
         }
       };
-      if (F == 2 && scattered_warp(x, y, z)) {
+      // x-pairs for scattered warps where a half's lights are more than its
+      // registers hold; with fewer lights the vote cost neighbouring pixels 4%
+      // (1080p x 32 lights 422 -> 400 us) and gave random points nothing (780
+      // -> 771), nor does it pay without the sampler
+      if (F == 2 && !HSMALL && !VIS && scattered_warp(x, y, z)) {
         if (a.table16)
           encode_half(a.table16, std::true_type{});
         else
@@ -517,7 +525,7 @@ __global__ void __launch_bounds__(2 * kTileM, MINB) fused_shade_pair_kernel(cons
 
       // ---- output layer: this half's lights -----------------------------------
       const float outmul = kF8 ? s_mult[a.n_layers - 1] : 1.0f;
-      if (V.vis_out) {
+      if constexpr (VIS) {
         for (int c0 = lo; c0 < hi; c0 += 16) {
           uint32_t r[16];
           tmem_ld16(t_lane + (uint32_t)c0, r);
@@ -1087,7 +1095,9 @@ size_t pair_smem(const nvc_handle* h, const PackArgs& p, FusedArgs* a = nullptr)
 template <int F, int PREC>
 cudaError_t launch_pair_typed(const FusedArgs& a, size_t smem_needed, int num_sms, cudaStream_t s) {
   const int H = split_h(a.L);
-  auto kern = H <= 16             ? fused_shade_pair_kernel<F, PREC, true, 3>
+  // a launch's views all export visibilities (nvc_infer) or none does
+  auto kern = a.v[0].vis_out      ? fused_shade_pair_kernel<F, PREC, true, 3, true>
+              : H <= 16           ? fused_shade_pair_kernel<F, PREC, true, 3>
               : a.tmem_cols > 128 ? fused_shade_pair_kernel<F, PREC, false, 2>
                                   : fused_shade_pair_kernel<F, PREC, false, 3>;
   const int max_ctas = (int)(512u / a.tmem_cols);
