@@ -592,9 +592,10 @@ static nvc_status shade_impl(nvc_handle* h, const nvc_scene* scene, const float*
     return NVC_OK;
   }
   StageScope sc(h, s, 3);
+  int launches = 0;
   NVC_CUDA(h, launch_shade_f32(h, scene, pos, nrm, n, seed, frame, view, pixel_offset, idx, pdf,
-                               wsum, radiance, s));
-  count_launches(h, 1);
+                               wsum, radiance, s, &launches));
+  count_launches(h, launches);
   return NVC_OK;
 }
 

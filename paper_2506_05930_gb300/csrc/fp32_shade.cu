@@ -367,7 +367,8 @@ cudaError_t launch_infer_f32(const nvc_handle* h, const float* pos, int64_t n, f
 cudaError_t launch_shade_f32(const nvc_handle* h, const nvc_scene* sc, const float* pos,
                              const float* nrm, int64_t n, uint64_t seed, uint32_t frame,
                              uint32_t view, int64_t pixel_offset, int32_t* idx, float* pdf,
-                             float* wsum, float* radiance, cudaStream_t s) {
+                             float* wsum, float* radiance, cudaStream_t s, int* launches) {
+  *launches = 0;
   if (n == 0) return cudaSuccess;
   ShadeArgs a = common_args(h, pos, n);
   a.nrm = nrm;
@@ -387,7 +388,10 @@ cudaError_t launch_shade_f32(const nvc_handle* h, const nvc_scene* sc, const flo
   // MLP 32-64-64-64-L, 578,731 pixels, on chip / staged (and the three-kernel
   // form before) in us: 32 lights 476 / 769 (1,395), 128 1,434 / 1,533
   // (2,999), 192 3,783 / 2,598 (4,094), 256 4,733 / 3,210 (4,771).
-  if (plan_smem(h, a.net, 4, true, nullptr) <= 227 * 1024) return launch<true>(a, h, s);
+  if (plan_smem(h, a.net, 4, true, nullptr) <= 227 * 1024) {
+    *launches = 1;
+    return launch<true>(a, h, s);
+  }
   const size_t smem = sizeof(float4) * ((h->L + 3) & ~3);
   for (int64_t o = 0; o < n; o += h->stage_pixels) {
     const int64_t m = n - o < h->stage_pixels ? n - o : h->stage_pixels;
@@ -398,6 +402,7 @@ cudaError_t launch_shade_f32(const nvc_handle* h, const nvc_scene* sc, const flo
         pixel_offset + o, idx ? idx + o : nullptr, pdf ? pdf + o : nullptr,
         wsum ? wsum + o : nullptr, radiance ? radiance + o : nullptr, a.neg0);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    *launches += 2;
   }
   return cudaSuccess;
 }

@@ -320,13 +320,14 @@ cudaError_t launch_wrs_from_weights(const float* w, int64_t n, int L, uint64_t s
                                     int32_t* idx, float* pdf, float* wsum, cudaStream_t s);
 
 // fp32_shade.cu: float32 inference, and inference + sampling + Neural DI, in
-// one kernel each.
+// one kernel each; *launches (the latter): kernels launched, one, or two per
+// staged chunk of a network whose outputs do not fit on chip.
 cudaError_t launch_infer_f32(const nvc_handle* h, const float* pos, int64_t n, float* vis,
                              cudaStream_t s);
 cudaError_t launch_shade_f32(const nvc_handle* h, const nvc_scene* sc, const float* pos,
                              const float* nrm, int64_t n, uint64_t seed, uint32_t frame,
                              uint32_t view, int64_t pixel_offset, int32_t* idx, float* pdf,
-                             float* wsum, float* radiance, cudaStream_t s);
+                             float* wsum, float* radiance, cudaStream_t s, int* launches);
 
 // fp32_train.cu: one float32 training pass (encode, forward, loss, backward,
 // scatter) in one kernel; false when the network does not fit on chip.
