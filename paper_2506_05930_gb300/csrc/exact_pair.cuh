@@ -69,6 +69,26 @@ __device__ __forceinline__ Pixel make_pixel(float px, float py, float pz, float 
   return p;
 }
 
+// sqrt(x) of both halves, correctly rounded for x of [2^-20, 2^64); nx = -x.
+__device__ __forceinline__ float2 sqrt2_rn(float2 x, float2 nx) {
+  float2 r;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r.x) : "f"(x.x));
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r.y) : "f"(x.y));
+  const float2 g = __fmul2_rn(x, r), h = __fmul2_rn(r, make_float2(-0.5f, -0.5f));
+  return __ffma2_rn(__ffma2_rn(g, g, nx), h, g);
+}
+
+// -(a / nb) of both halves, correctly rounded while nothing leaves the normal
+// range.
+__device__ __forceinline__ float2 div2_rn(float2 a, float2 nb) {
+  float2 y;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y.x) : "f"(-nb.x));
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y.y) : "f"(-nb.y));
+  y = __ffma2_rn(__ffma2_rn(nb, y, make_float2(1.0f, 1.0f)), y, y);
+  const float2 q = __fmul2_rn(a, y);
+  return __ffma2_rn(__ffma2_rn(nb, q, a), y, q);
+}
+
 // Two contributions; dmin and tmin collect what the bounds check: the least
 // |d|^2, and the least positive numerator (bits - 1, so that zero and
 // negative ones, whose contribution is 0, come out largest).
@@ -81,19 +101,10 @@ __device__ __forceinline__ float2 contribution2(const Pixel& p, float4 A, float4
                                __ffma2_rn(dz, dz, p.neg0));
   const float2 ndl = __fadd2_rn(__fadd2_rn(__ffma2_rn(p.nx, dx, p.neg0), __ffma2_rn(p.ny, dy, p.neg0)),
                                 __ffma2_rn(p.nz, dz, p.neg0));
-  float2 r, y;
-  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r.x) : "f"(d2.x));
-  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r.y) : "f"(d2.y));
   const float2 nd2 = __fmul2_rn(d2, make_float2(-1.0f, -1.0f));
-  const float2 g = __fmul2_rn(d2, r), h = __fmul2_rn(r, make_float2(-0.5f, -0.5f));
-  const float2 s = __ffma2_rn(__ffma2_rn(g, g, nd2), h, g);       // sqrt(d2)
-  const float2 nden = __fmul2_rn(s, nd2);                         // -sqrt(d2) d2, d2 >= 1e-6
+  const float2 nden = __fmul2_rn(sqrt2_rn(d2, nd2), nd2);         // -sqrt(d2) d2, d2 >= 1e-6
   const float2 num = __fmul2_rn(make_float2(B.z, B.w), ndl);
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y.x) : "f"(-nden.x));
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y.y) : "f"(-nden.y));
-  y = __ffma2_rn(__ffma2_rn(nden, y, make_float2(1.0f, 1.0f)), y, y);
-  const float2 q = __fmul2_rn(num, y);
-  const float2 c = __ffma2_rn(__ffma2_rn(nden, q, num), y, q);    // num / den
+  const float2 c = div2_rn(num, nden);                            // num / den
   dmin = fminf(fminf(dmin, d2.x), d2.y);
   tmin = min(min(tmin, __float_as_uint(num.x) - 1u), __float_as_uint(num.y) - 1u);
   return make_float2(fmaxf(c.x, 0.0f), fmaxf(c.y, 0.0f));   // n.d <= 0 (or NaN) gives 0
