@@ -51,6 +51,7 @@ __device__ __forceinline__ int member_of(const int32_t* off, const int32_t* mem,
   return mem[off[y] + (int)(((uint64_t)r * m) >> 32)];
 }
 
+template <bool FEW>
 __global__ void __launch_bounds__(256) cluster_targets_kernel(
     const float* __restrict__ lights, const float* __restrict__ spheres, int n_sph,
     const float* __restrict__ boxes, int n_box, const int32_t* __restrict__ off,
@@ -58,7 +59,7 @@ __global__ void __launch_bounds__(256) cluster_targets_kernel(
     uint32_t k0, uint32_t k1, uint32_t frame, float* __restrict__ target) {
   extern __shared__ float4 s_occ[];
   const Occluders occ =
-      stage_occluders(spheres, n_sph, boxes, n_box, s_occ, threadIdx.x, blockDim.x);
+      stage_occluders<FEW>(spheres, n_sph, boxes, n_box, s_occ, threadIdx.x, blockDim.x);
   __syncthreads();
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= n * k) return;
@@ -69,7 +70,7 @@ __global__ void __launch_bounds__(256) cluster_targets_kernel(
     const int x = member_of(off, mem, y, stream_word((uint32_t)b, frame, 0u, kTagCluster, y, k0, k1));
     const float4 l = reinterpret_cast<const float4*>(lights)[x];
     const float px = pos[3 * b], py = pos[3 * b + 1], pz = pos[3 * b + 2];
-    v = segment_blocked(px, py, pz, l.x, l.y, l.z, occ) ? 0.0f : 1.0f;
+    v = segment_blocked<FEW>(px, py, pz, l.x, l.y, l.z, occ) ? 0.0f : 1.0f;
   }
   target[t] = v;
 }
@@ -166,7 +167,7 @@ struct ClusterArgs {
 // of cluster y (y < 0: nothing contributes) with weight w_y of wsum, the
 // unbiased contribution weight, and the one-ray estimate.  light(slot): the
 // light at a place of the cluster table, I / pi in w.
-template <typename LightFn>
+template <bool FEW, typename LightFn>
 __device__ __forceinline__ void finish_pixel(const ClusterArgs& a, int64_t p, int y, float w_y,
                                              float wsum, int base, uint32_t m_y, float px, float py,
                                              float pz, xp::Pixel pp, LightFn light,
@@ -219,7 +220,7 @@ __device__ __forceinline__ void finish_pixel(const ClusterArgs& a, int64_t p, in
     float e = 0.0f;
     if (sel_light >= 0) {
       const float4 l = reinterpret_cast<const float4*>(a.lights)[sel_light];
-      if (!segment_blocked(px, py, pz, l.x, l.y, l.z, occ)) e = __fmul_rn(cx, W);
+      if (!segment_blocked<FEW>(px, py, pz, l.x, l.y, l.z, occ)) e = __fmul_rn(cx, W);
     }
     a.estimate[p] = e;
   }
@@ -235,12 +236,14 @@ __device__ __forceinline__ float4 table_light(const ClusterArgs& a, int slot) {
 // ---- first-step weights max(v, 0.001) alone ---------------------------------
 // No light loop: a pixel's visibilities are loaded together (16-byte loads
 // when the row allows) into the weights' registers.
+template <bool FEW>
 __global__ void __launch_bounds__(128, 7) sample_visibility_kernel(const __grid_constant__ ClusterArgs a,
                                                                  bool vis_vec4) {
   extern __shared__ float4 s_scene4[];
   int32_t* s_off = reinterpret_cast<int32_t*>(s_scene4);
-  const Occluders occ = stage_occluders(a.spheres, a.n_sph, a.boxes, a.n_box,
-                                        s_scene4 + (kMaxClusters + 4) / 4, threadIdx.x, blockDim.x);
+  const Occluders occ = stage_occluders<FEW>(a.spheres, a.n_sph, a.boxes, a.n_box,
+                                             s_scene4 + (kMaxClusters + 4) / 4, threadIdx.x,
+                                             blockDim.x);
   const int k = a.k;
   for (int e = threadIdx.x; e <= k; e += blockDim.x) s_off[e] = a.off[e];
   __syncthreads();
@@ -281,7 +284,7 @@ __global__ void __launch_bounds__(128, 7) sample_visibility_kernel(const __grid_
     for (int t = 0; t < kMaxClusters; ++t)
       if (t == y) w_y = w[t];
     const int base = y < 0 ? 0 : s_off[y];
-    finish_pixel(a, p, y, w_y, wsum, base, y < 0 ? 0u : (uint32_t)(s_off[y + 1] - base), px, py, pz,
+    finish_pixel<FEW>(a, p, y, w_y, wsum, base, y < 0 ? 0u : (uint32_t)(s_off[y + 1] - base), px, py, pz,
                  xp::make_pixel(px, py, pz, nx, ny, nz, a.neg0, true),
                  [&](int slot) { return table_light(a, slot); }, occ);
   }
@@ -326,6 +329,7 @@ __device__ __forceinline__ bool stage_slots(const ClusterArgs& a, const int32_t*
   return ok;
 }
 
+template <bool FEW>
 __global__ void __launch_bounds__(kSumThreads, 3)
     sample_sum_kernel(const __grid_constant__ ClusterArgs a) {
   extern __shared__ float4 s_scene4[];
@@ -333,8 +337,8 @@ __global__ void __launch_bounds__(kSumThreads, 3)
   float* s_w = reinterpret_cast<float*>(s_lt + a.tile) + threadIdx.x;
   int32_t* s_off = reinterpret_cast<int32_t*>(s_lt + a.tile) + kMaxClusters * kSumThreads;
   int32_t* s_pad = s_off + kMaxClusters + 4;
-  const Occluders occ = stage_occluders(a.spheres, a.n_sph, a.boxes, a.n_box,
-                                        s_pad + kMaxClusters + 4, threadIdx.x, blockDim.x);
+  const Occluders occ = stage_occluders<FEW>(a.spheres, a.n_sph, a.boxes, a.n_box,
+                                             s_pad + kMaxClusters + 4, threadIdx.x, blockDim.x);
   const int k = a.k;
   for (int e = threadIdx.x; e <= k; e += blockDim.x) s_off[e] = a.off[e];
   __syncthreads();
@@ -404,7 +408,7 @@ __global__ void __launch_bounds__(kSumThreads, 3)
                           (uint32_t)(a.pixel_offset + p), a.frame, a.view, a.k0, a.k1);
     const int base = y < 0 ? 0 : s_off[y];
     pp.ok = pixel_ok;
-    finish_pixel(a, p, y, y < 0 ? 0.0f : s_w[y * kSumThreads], wsum, base,
+    finish_pixel<FEW>(a, p, y, y < 0 ? 0.0f : s_w[y * kSumThreads], wsum, base,
                  y < 0 ? 0u : (uint32_t)(s_off[y + 1] - base), px, py, pz, pp,
                  [&](int slot) {
                    return whole ? xp::pair_light(s_lt, s_pad[y] + slot - base) : table_light(a, slot);
@@ -426,6 +430,7 @@ __device__ __forceinline__ float target_of(const float* lights, int n_lights, in
   return contribution(px, py, pz, nx, ny, nz, l.x, l.y, l.z, __fmul_rn(l.w, bits_f(kInvPiBits)));
 }
 
+template <bool FEW>
 __global__ void __launch_bounds__(256) temporal_merge_kernel(
     const float* __restrict__ lights, int n_lights, const float* __restrict__ spheres, int n_sph,
     const float* __restrict__ boxes, int n_box, const float* __restrict__ pos,
@@ -438,7 +443,7 @@ __global__ void __launch_bounds__(256) temporal_merge_kernel(
   extern __shared__ float4 s_occ[];
   Occluders occ = no_occluders(s_occ);
   if (estimate) {
-    occ = stage_occluders(spheres, n_sph, boxes, n_box, s_occ, threadIdx.x, blockDim.x);
+    occ = stage_occluders<FEW>(spheres, n_sph, boxes, n_box, s_occ, threadIdx.x, blockDim.x);
     __syncthreads();
   }
   for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < n;
@@ -471,7 +476,8 @@ __global__ void __launch_bounds__(256) temporal_merge_kernel(
       float e = 0.0f;
       if (y >= 0) {
         const float4 l = __ldg(reinterpret_cast<const float4*>(lights) + y);
-        if (!segment_blocked(px, py, pz, l.x, l.y, l.z, occ)) e = __fmul_rn(j == 0 ? pc : pp, W);
+        if (!segment_blocked<FEW>(px, py, pz, l.x, l.y, l.z, occ))
+          e = __fmul_rn(j == 0 ? pc : pp, W);
       }
       estimate[p] = e;
     }
@@ -488,14 +494,13 @@ cudaError_t launch_temporal_merge(const nvc_scene* sc, const float* pos, const f
                                   float* estimate, int num_sms, cudaStream_t s) {
   if (n == 0) return cudaSuccess;
   const size_t smem = estimate ? occluder_bytes(sc->n_spheres, sc->n_boxes) : 0;
-  if (smem > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(temporal_merge_kernel,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-  }
+  auto kern = few_occluders(sc->n_spheres, sc->n_boxes) ? temporal_merge_kernel<true>
+                                                        : temporal_merge_kernel<false>;
+  const cudaError_t e = allow_smem(kern, smem);
+  if (e != cudaSuccess) return e;
   const int64_t want = (n + 255) / 256;
   const int64_t cap = (int64_t)num_sms * 8;
-  temporal_merge_kernel<<<(unsigned)(want < cap ? want : cap), 256, smem, s>>>(
+  kern<<<(unsigned)(want < cap ? want : cap), 256, smem, s>>>(
       sc->lights, sc->n_lights, sc->spheres, sc->n_spheres, sc->boxes, sc->n_boxes, pos, nrm, n,
       pixel_offset, (uint32_t)seed, (uint32_t)(seed >> 32), frame, view, cur_light, cur_W,
       prev_light, prev_W, prev_M, light, W, M, estimate);
@@ -508,9 +513,11 @@ cudaError_t launch_cluster_targets(const nvc_scene* sc, const nvc_clusters* cl, 
   if (n == 0) return cudaSuccess;
   const int64_t total = n * cl->k;
   const size_t smem = occluder_bytes(sc->n_spheres, sc->n_boxes);
-  const cudaError_t e = allow_smem(cluster_targets_kernel, smem);
+  auto kern = few_occluders(sc->n_spheres, sc->n_boxes) ? cluster_targets_kernel<true>
+                                                        : cluster_targets_kernel<false>;
+  const cudaError_t e = allow_smem(kern, smem);
   if (e != cudaSuccess) return e;
-  cluster_targets_kernel<<<(unsigned)((total + 255) / 256), 256, smem, s>>>(
+  kern<<<(unsigned)((total + 255) / 256), 256, smem, s>>>(
       sc->lights, sc->spheres, sc->n_spheres, sc->boxes, sc->n_boxes, cl->offsets, cl->members,
       cl->k, pos, n, (uint32_t)seed, (uint32_t)(seed >> 32), frame, target);
   return cudaGetLastError();
@@ -543,7 +550,10 @@ cudaError_t launch_sample_clustered(const nvc_scene* sc, const nvc_clusters* cl,
                       (uint32_t)seed, (uint32_t)(seed >> 32), frame, view, light, weight, estimate,
                       -0.0f, light_slots(sc, cl)};
   const bool sum = cl->weights != NVC_CLUSTER_WEIGHT_VISIBILITY;
-  const void* kern = sum ? (const void*)sample_sum_kernel : (const void*)sample_visibility_kernel;
+  const bool few = few_occluders(sc->n_spheres, sc->n_boxes);
+  auto sum_kern = few ? sample_sum_kernel<true> : sample_sum_kernel<false>;
+  auto vis_kern = few ? sample_visibility_kernel<true> : sample_visibility_kernel<false>;
+  const void* kern = sum ? (const void*)sum_kern : (const void*)vis_kern;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   // one wave of resident CTAs strides over the pixels
@@ -555,11 +565,11 @@ cudaError_t launch_sample_clustered(const nvc_scene* sc, const nvc_clusters* cl,
   const int64_t want = (n + threads - 1) / threads, cap = (int64_t)num_sms * per_sm;
   const int grid = (int)(want < cap ? want : cap);
   if (sum) {
-    sample_sum_kernel<<<grid, threads, smem, s>>>(a);
+    sum_kern<<<grid, threads, smem, s>>>(a);
   } else {
     // 16-byte loads of a pixel's visibilities need rows of a multiple of 4
     // floats on a 16-byte aligned base
-    sample_visibility_kernel<<<grid, threads, smem, s>>>(
+    vis_kern<<<grid, threads, smem, s>>>(
         a, (cl->k & 3) == 0 && (reinterpret_cast<uintptr_t>(vis) & 15) == 0);
   }
   return cudaGetLastError();

@@ -22,6 +22,7 @@ namespace nvc {
 
 namespace {
 
+template <bool FEW>
 __global__ void __launch_bounds__(256) shade_estimate_kernel(
     const float* __restrict__ lights, const float* __restrict__ spheres, int n_sph,
     const float* __restrict__ boxes, int n_box, const float* __restrict__ pos,
@@ -30,7 +31,7 @@ __global__ void __launch_bounds__(256) shade_estimate_kernel(
     uint32_t count) {
   extern __shared__ float4 s_scene4[];
   const Occluders occ =
-      stage_occluders(spheres, n_sph, boxes, n_box, s_scene4, threadIdx.x, blockDim.x);
+      stage_occluders<FEW>(spheres, n_sph, boxes, n_box, s_scene4, threadIdx.x, blockDim.x);
   __syncthreads();
   for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < n;
        p += (int64_t)gridDim.x * blockDim.x) {
@@ -42,7 +43,7 @@ __global__ void __launch_bounds__(256) shade_estimate_kernel(
       const float px = pos[3 * p], py = pos[3 * p + 1], pz = pos[3 * p + 2];
       const float c = contribution(px, py, pz, nrm[3 * p], nrm[3 * p + 1], nrm[3 * p + 2], l.x,
                                    l.y, l.z, __fmul_rn(l.w, bits_f(kInvPiBits)));
-      if (c > 0.0f && !segment_blocked(px, py, pz, l.x, l.y, l.z, occ))
+      if (c > 0.0f && !segment_blocked<FEW>(px, py, pz, l.x, l.y, l.z, occ))
         e = __fdiv_rn(c, pr);
     }
     if (estimate) estimate[p] = e;
@@ -142,6 +143,48 @@ __global__ void __launch_bounds__(256, 3) exact_di_kernel(
   }
 }
 
+// Few occluders: a light at a time for each pixel by itself.  The warp's vote,
+// the packed contributions and 80 registers a thread cost more there than they
+// save.  130,000 pixels x 32 lights, this kernel / the one above in us:
+// no occluder 12 / 23, 4 spheres 35 / 55, 8 boxes 53 / 57, 6 + 6 78 / 74
+// (random positions 78 / 99), 8 + 8 94 / 84 (96 / 111).
+template <bool kSmemLights>
+__global__ void __launch_bounds__(256) exact_di_few_kernel(
+    const float* __restrict__ lights, int L, const float* __restrict__ spheres, int n_sph,
+    const float* __restrict__ boxes, int n_box, const float* __restrict__ pos,
+    const float* __restrict__ nrm, int64_t n, float* __restrict__ di, float) {
+  extern __shared__ float4 s_scene4[];
+  const Occluders occ = stage_occluders<true>(spheres, n_sph, boxes, n_box,
+                                              s_scene4 + (kSmemLights ? (L + 3) & ~3 : 0),
+                                              threadIdx.x, blockDim.x);
+  if (kSmemLights) {
+    for (int e = threadIdx.x; e < L; e += blockDim.x) {
+      float4 l = reinterpret_cast<const float4*>(lights)[e];
+      l.w = __fmul_rn(l.w, bits_f(kInvPiBits));
+      s_scene4[e] = l;
+    }
+  }
+  __syncthreads();
+  for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < n;
+       p += (int64_t)gridDim.x * blockDim.x) {
+    const float px = pos[3 * p], py = pos[3 * p + 1], pz = pos[3 * p + 2];
+    const float nx = nrm[3 * p], ny = nrm[3 * p + 1], nz = nrm[3 * p + 2];
+    float sum = 0.0f;
+    for (int i = 0; i < L; ++i) {
+      float4 l;
+      if (kSmemLights) {
+        l = s_scene4[i];
+      } else {
+        l = __ldg(reinterpret_cast<const float4*>(lights) + i);
+        l.w = __fmul_rn(l.w, bits_f(kInvPiBits));
+      }
+      const float c = contribution(px, py, pz, nx, ny, nz, l.x, l.y, l.z, l.w);
+      if (c > 0.0f && !segment_blocked<true>(px, py, pz, l.x, l.y, l.z, occ)) sum = __fadd_rn(sum, c);
+    }
+    di[p] = sum;
+  }
+}
+
 int grid_for(int64_t n, int num_sms) {
   const int64_t want = (n + 255) / 256;
   const int64_t cap = (int64_t)num_sms * 8;
@@ -156,9 +199,11 @@ cudaError_t launch_shade_estimate(const nvc_scene* sc, const float* pos, const f
                                   cudaStream_t s) {
   if (n == 0) return cudaSuccess;
   const size_t smem = occluder_bytes(sc->n_spheres, sc->n_boxes);
-  const cudaError_t e = allow_smem(shade_estimate_kernel, smem);
+  auto kern = few_occluders(sc->n_spheres, sc->n_boxes) ? shade_estimate_kernel<true>
+                                                        : shade_estimate_kernel<false>;
+  const cudaError_t e = allow_smem(kern, smem);
   if (e != cudaSuccess) return e;
-  shade_estimate_kernel<<<grid_for(n, num_sms), 256, smem, s>>>(
+  kern<<<grid_for(n, num_sms), 256, smem, s>>>(
       sc->lights, sc->spheres, sc->n_spheres, sc->boxes, sc->n_boxes, pos, nrm, n, idx, pdf,
       estimate, accum, count);
   return cudaGetLastError();
@@ -171,7 +216,9 @@ cudaError_t launch_exact_di(const nvc_scene* sc, const float* pos, const float* 
   const size_t lt = sizeof(float) * 4 * (((size_t)sc->n_lights + 3) & ~(size_t)3);
   const bool on_chip = occ + lt <= 227 * 1024;
   const size_t smem = on_chip ? occ + lt : occ;
-  auto kern = on_chip ? exact_di_kernel<true> : exact_di_kernel<false>;
+  const bool few = sc->n_spheres + sc->n_boxes <= 12;
+  auto kern = few ? (on_chip ? exact_di_few_kernel<true> : exact_di_few_kernel<false>)
+                  : (on_chip ? exact_di_kernel<true> : exact_di_kernel<false>);
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   kern<<<grid_for(n, num_sms), 256, smem, s>>>(sc->lights, sc->n_lights, sc->spheres,

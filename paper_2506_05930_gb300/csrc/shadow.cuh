@@ -21,13 +21,23 @@ namespace nvc {
 //   slab test reads the box itself from the scene's array.
 // The pairs are held against a segment two occluders at a time (near_spheres,
 // near_boxes), and what stands is tested exactly one by one.
+// FEW (few_occluders): every test is exact, and the boxes are staged as they
+// are, 24 bytes each: (lo_x, hi_x), (lo_y, hi_y), (lo_z, hi_z).
 struct Occluders {
   const float4* sph;   // 2 float4 per sphere pair
   int n_pairs;
-  const float4* box;   // 3 float4 per box pair
+  const float4* box;   // 3 float4 per box pair; FEW: 3 float2 per box
   int n_box;
   const float* boxes;  // the scene's boxes, lo and hi (global memory)
 };
+
+// Whether a scene's rays take the FEW kernels.  Dropping occluders by pairs
+// first costs a ray some 40 operations and its kernel 16 registers a thread
+// (48 against 32: 40 warps an SM against 64), which few exact tests do not pay
+// back; a sphere's test is about three times a box's.  130,000 points x 32
+// lights, FEW / other in us: 4 spheres 32.8 / 45.2, 4 boxes 32.8 / 49.2, 8 + 8
+// 77.3 / 84.0, 12 + 12 102.6 / 100.4, 16 + 16 129 / 117.
+inline bool few_occluders(int n_sph, int n_box) { return 3 * n_sph + n_box <= 36; }
 
 __host__ __device__ __forceinline__ size_t occluder_bytes(int n_sph, int n_box) {
   return 32 * (size_t)((n_sph + 1) / 2) + 48 * (size_t)((n_box + 1) / 2);
@@ -35,6 +45,7 @@ __host__ __device__ __forceinline__ size_t occluder_bytes(int n_sph, int n_box) 
 
 // Stages the occluders at dst (16-byte aligned; occluder_bytes(...) long),
 // threads tid of nthreads sharing the work; the caller synchronises.
+template <bool FEW = false>
 __device__ __forceinline__ Occluders stage_occluders(const float* __restrict__ spheres, int n_sph,
                                                      const float* __restrict__ boxes, int n_box,
                                                      void* dst, int tid, int nthreads) {
@@ -56,17 +67,27 @@ __device__ __forceinline__ Occluders stage_occluders(const float* __restrict__ s
     q[6] = sp.w;
   }
   float* b = f + 8 * o.n_pairs;
-  for (int e = tid; e < ((n_box + 1) & ~1); e += nthreads) {
-    float* q = b + 12 * (e >> 1) + (e & 1);
+  if constexpr (FEW) {
+    for (int e = tid; e < n_box; e += nthreads) {
 #pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      float lo = 0.0f, hi = 0.0f;   // an odd count's last slot: never read as a box
-      if (e < n_box) {
-        lo = boxes[6 * e + a];
-        hi = boxes[6 * e + 3 + a];
+      for (int a = 0; a < 3; ++a) {
+        b[6 * e + 2 * a] = boxes[6 * e + a];
+        b[6 * e + 2 * a + 1] = boxes[6 * e + 3 + a];
       }
-      q[4 * a] = 0.5f * lo + 0.5f * hi;
-      q[4 * a + 2] = fabsf(0.5f * hi - 0.5f * lo) + 0x1p-16f * (fabsf(lo) + fabsf(hi));
+    }
+  } else {
+    for (int e = tid; e < ((n_box + 1) & ~1); e += nthreads) {
+      float* q = b + 12 * (e >> 1) + (e & 1);
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        float lo = 0.0f, hi = 0.0f;   // an odd count's last slot: never read as a box
+        if (e < n_box) {
+          lo = boxes[6 * e + a];
+          hi = boxes[6 * e + 3 + a];
+        }
+        q[4 * a] = 0.5f * lo + 0.5f * hi;
+        q[4 * a + 2] = fabsf(0.5f * hi - 0.5f * lo) + 0x1p-16f * (fabsf(lo) + fabsf(hi));
+      }
     }
   }
   o.box = reinterpret_cast<const float4*>(b);
@@ -281,11 +302,47 @@ __device__ __forceinline__ uint32_t near_boxes(const Segment& g, const Occluders
   return 2 * k1 > occ.n_box ? m & ~(1u << (occ.n_box - 2 * k0)) : m;   // not the padding slot
 }
 
+// segment_blocked of the FEW kernels: every occluder tested exactly, with the
+// reciprocals that the scene's kinds of occluders need.
+__device__ __forceinline__ bool segment_blocked_few(float px, float py, float pz, float lx, float ly,
+                                                    float lz, const Occluders& occ) {
+  const float dx = __fsub_rn(lx, px), dy = __fsub_rn(ly, py), dz = __fsub_rn(lz, pz);
+  bool blocked = false;
+  if (occ.n_pairs > 0) {
+    const float dd = dot3_rn(dx, dy, dz, dx, dy, dz);
+    // a zero-length segment (light on the point): t stays at t0
+    const float inv_dd = dd > 0.0f ? rcp_rn(dd) : 0.0f;
+    for (int k = 0; k < occ.n_pairs && !blocked; ++k) {
+      const float4 A = occ.sph[2 * k], B = occ.sph[2 * k + 1];
+      blocked = sphere_lane_blocks(px, py, pz, dx, dy, dz, inv_dd, A.x, A.z, B.x, B.z) ||
+                sphere_lane_blocks(px, py, pz, dx, dy, dz, inv_dd, A.y, A.w, B.y, B.w);
+    }
+  }
+  if (occ.n_box > 0 && !blocked) {
+    const float2* b = reinterpret_cast<const float2*>(occ.box);
+    const float ix = dx != 0.0f ? rcp_rn(dx) : 0.0f;
+    const float iy = dy != 0.0f ? rcp_rn(dy) : 0.0f;
+    const float iz = dz != 0.0f ? rcp_rn(dz) : 0.0f;
+    if (dx != 0.0f && dy != 0.0f && dz != 0.0f) {
+      const float2 px2 = make_float2(px, px), py2 = make_float2(py, py), pz2 = make_float2(pz, pz);
+      const float2 ix2 = make_float2(ix, ix), iy2 = make_float2(iy, iy), iz2 = make_float2(iz, iz);
+      for (int k = 0; k < occ.n_box && !blocked; ++k)
+        blocked = box_blocks_oblique(px2, py2, pz2, ix2, iy2, iz2, b + 3 * k);
+    } else {
+      for (int k = 0; k < occ.n_box && !blocked; ++k)
+        blocked = box_blocks_general(px, py, pz, dx, dy, dz, ix, iy, iz, b + 3 * k);
+    }
+  }
+  return blocked;
+}
+
 // Whether the segment from (px, py, pz) to the light at (lx, ly, lz) is
-// blocked by one of the staged occluders: those that near_spheres and
-// near_boxes keep are tested exactly.
+// blocked by one of the staged occluders (staged with the same FEW): those
+// that near_spheres and near_boxes keep are tested exactly.
+template <bool FEW = false>
 __device__ __forceinline__ bool segment_blocked(float px, float py, float pz, float lx, float ly,
                                                 float lz, const Occluders& occ) {
+  if constexpr (FEW) return segment_blocked_few(px, py, pz, lx, ly, lz, occ);
   const Segment g = make_segment(px, py, pz, lx, ly, lz);
   const float slack = 0x1p-15f * (px * px + py * py + pz * pz + lx * lx + ly * ly + lz * lz);
   bool blocked = false;

@@ -20,14 +20,14 @@ __global__ void training_positions_kernel(PosGen g, int64_t batch, float* __rest
 // ---- shadow rays (occluder tests in shadow.cuh) -------------------------------
 // GEN: the kernel also makes the training positions (training_position),
 // the lane of light 0 storing each; otherwise it reads them from pos.
-template <bool GEN>
+template <bool GEN, bool FEW>
 __global__ void __launch_bounds__(256) trace_visibility_kernel(
     const float* __restrict__ lights, int L, const float* __restrict__ spheres, int n_sph,
     const float* __restrict__ boxes, int n_box, float* __restrict__ pos, int64_t n,
     float* __restrict__ vis, PosGen gen) {
   extern __shared__ float4 s_occ[];
   const Occluders occ =
-      stage_occluders(spheres, n_sph, boxes, n_box, s_occ, threadIdx.x, blockDim.x);
+      stage_occluders<FEW>(spheres, n_sph, boxes, n_box, s_occ, threadIdx.x, blockDim.x);
   __syncthreads();
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= n * L) return;
@@ -50,7 +50,7 @@ __global__ void __launch_bounds__(256) trace_visibility_kernel(
     pz = pos[3 * p + 2];
   }
   const float4 lt = reinterpret_cast<const float4*>(lights)[i];
-  const bool blocked = segment_blocked(px, py, pz, lt.x, lt.y, lt.z, occ);
+  const bool blocked = segment_blocked<FEW>(px, py, pz, lt.x, lt.y, lt.z, occ);
   vis[t] = blocked ? 0.0f : 1.0f;
 }
 
@@ -417,9 +417,11 @@ cudaError_t launch_training_data(const nvc_scene* sc, const float* screen_pos, i
     return launch_training_positions(sc, screen_pos, n_screen, batch, seed, frame, pos, s, n_world);
   const int64_t total = batch * sc->n_lights;
   const size_t smem = occluder_bytes(sc->n_spheres, sc->n_boxes);
-  const cudaError_t e = allow_smem(trace_visibility_kernel<true>, smem);
+  auto kern = few_occluders(sc->n_spheres, sc->n_boxes) ? trace_visibility_kernel<true, true>
+                                                        : trace_visibility_kernel<true, false>;
+  const cudaError_t e = allow_smem(kern, smem);
   if (e != cudaSuccess) return e;
-  trace_visibility_kernel<true><<<(unsigned)((total + 255) / 256), 256, smem, s>>>(
+  kern<<<(unsigned)((total + 255) / 256), 256, smem, s>>>(
       sc->lights, sc->n_lights, sc->spheres, sc->n_spheres, sc->boxes, sc->n_boxes, pos, batch,
       vis, pos_gen(sc, screen_pos, n_screen, batch, seed, frame, n_world));
   return cudaGetLastError();
@@ -430,9 +432,11 @@ cudaError_t launch_trace_visibility(const nvc_scene* sc, const float* pos, int64
   if (n == 0) return cudaSuccess;
   const int64_t total = n * sc->n_lights;
   const size_t smem = occluder_bytes(sc->n_spheres, sc->n_boxes);
-  const cudaError_t e = allow_smem(trace_visibility_kernel<false>, smem);
+  auto kern = few_occluders(sc->n_spheres, sc->n_boxes) ? trace_visibility_kernel<false, true>
+                                                        : trace_visibility_kernel<false, false>;
+  const cudaError_t e = allow_smem(kern, smem);
   if (e != cudaSuccess) return e;
-  trace_visibility_kernel<false><<<(unsigned)((total + 255) / 256), 256, smem, s>>>(
+  kern<<<(unsigned)((total + 255) / 256), 256, smem, s>>>(
       sc->lights, sc->n_lights, sc->spheres, sc->n_spheres, sc->boxes, sc->n_boxes,
       const_cast<float*>(pos), n, vis, PosGen{});
   return cudaGetLastError();
