@@ -56,9 +56,11 @@ __global__ void __launch_bounds__(256) shade_estimate_kernel(
 
 // One light at a time for the whole warp (warp_segments_blocked), its
 // contribution two lights per packed operation (exact_pair.cuh).  A warp whose
-// pixels are not neighbours -- its first light's vote keeps more than half of
-// the occluders -- takes segment_blocked for the rest of its lights, so the
-// votes cost it one light.
+// pixels are not neighbours -- a light's vote keeps more than an eighth of the
+// occluders -- takes segment_blocked from there on, so the votes cost it one
+// ballot a 32 occluders (a million pixels x 8 lights, 32 + 32: 128 us, with the
+// limit at a half and the kept ones tested first 147; random positions 395 and
+// 457; 4,096 pixels x 32 lights, 500 + 500: 340 and 1,008).
 // 1920x1080 x 32 lights, 32 spheres + 32 boxes: 2.80 -> 0.757 ms; bound by
 // instruction issue (9,900 a warp and 32 lights; 75% of the slots).
 // kSmemLights: the lights (with I / pi) are staged after the occluders as
@@ -85,7 +87,7 @@ __global__ void __launch_bounds__(256, 3) exact_di_kernel(
     }
   }
   lights_ok = __syncthreads_and(lights_ok) != 0;
-  const int n_occ = 2 * occ.n_pairs + occ.n_box;
+  const int limit = (2 * occ.n_pairs + occ.n_box) / 8 + 2;
   // whole warps walk the pixels: a lane past the end repeats the warp's first
   // pixel and writes nothing
   for (int64_t p0 = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); p0 < n;
@@ -129,13 +131,9 @@ __global__ void __launch_bounds__(256, 3) exact_di_kernel(
         const bool want = live && i0 + q < L && cq > 0.0f;
         if (!__any_sync(0xffffffffu, want)) continue;
         bool blocked = false;
-        if (together) {
-          int tested = 0;
-          blocked = warp_segments_blocked(hull, want, px, py, pz, l.x, l.y, l.z, occ, &tested);
-          together = 2 * tested <= n_occ;
-        } else if (want) {
-          blocked = segment_blocked(px, py, pz, l.x, l.y, l.z, occ);
-        }
+        if (together)
+          together = warp_segments_blocked(hull, want, px, py, pz, l.x, l.y, l.z, occ, limit, &blocked);
+        if (!together && want) blocked = segment_blocked(px, py, pz, l.x, l.y, l.z, occ);
         if (want && !blocked) sum = __fadd_rn(sum, cq);
       }
     }

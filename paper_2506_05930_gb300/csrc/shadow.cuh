@@ -455,33 +455,37 @@ __device__ __forceinline__ bool hull_meets_box(const WarpHull& w, const HullRay&
   return !(tmin > tmax);
 }
 
-// segment_blocked for a whole warp looking at one light: the lanes with
-// `want` get their answer, the others false.  *tested (the same in all lanes)
-// grows by the exact tests taken.
+// segment_blocked for a whole warp looking at one light: *blocked is the
+// answer of the lanes with `want`.  Gives up, with false in every lane, when
+// more than `limit` occluders would have to be tested exactly.
 __device__ __forceinline__ bool warp_segments_blocked(const WarpHull& w, bool want, float px, float py,
                                                       float pz, float lx, float ly, float lz,
-                                                      const Occluders& occ, int* tested) {
+                                                      const Occluders& occ, int limit, bool* blocked) {
   const int lane = threadIdx.x & 31;
   const HullRay r = hull_ray(w, lx, ly, lz);
   const Segment g = make_segment(px, py, pz, lx, ly, lz);
   bool open = want;
+  *blocked = want;   // until the last occluder is past with lanes still open
   for (int b = 0; b < 2 * occ.n_pairs; b += 32) {
     const bool near = b + lane < 2 * occ.n_pairs && hull_meets_sphere(w, r, occ, b + lane);
-    for (unsigned m = __ballot_sync(0xffffffffu, near); m; m &= m - 1) {
+    unsigned m = __ballot_sync(0xffffffffu, near);
+    if ((limit -= __popc(m)) < 0) return false;
+    for (; m; m &= m - 1) {
       open = open && !sphere_blocks(g, occ, b + __ffs(m) - 1);
-      ++*tested;
-      if (!__any_sync(0xffffffffu, open)) return want;
+      if (!__any_sync(0xffffffffu, open)) return true;
     }
   }
   for (int b = 0; b < occ.n_box; b += 32) {
     const bool near = b + lane < occ.n_box && hull_meets_box(w, r, occ, b + lane);
-    for (unsigned m = __ballot_sync(0xffffffffu, near); m; m &= m - 1) {
+    unsigned m = __ballot_sync(0xffffffffu, near);
+    if ((limit -= __popc(m)) < 0) return false;
+    for (; m; m &= m - 1) {
       open = open && !box_blocks(g, occ, b + __ffs(m) - 1);
-      ++*tested;
-      if (!__any_sync(0xffffffffu, open)) return want;
+      if (!__any_sync(0xffffffffu, open)) return true;
     }
   }
-  return want && !open;
+  *blocked = want && !open;
+  return true;
 }
 
 // ---- training positions (Section 3.4) ------------------------------------------
