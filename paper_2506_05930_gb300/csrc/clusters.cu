@@ -308,11 +308,11 @@ __global__ void __launch_bounds__(128, 7) sample_visibility_kernel(const __grid_
 constexpr int kLightTile = 1024;
 constexpr int kSumThreads = 256;
 
-// Light slots [t0, t0 + tn) of the padded table into s_lt; whether this
-// thread's lights are inside the packed contribution's bounds.
-__device__ __forceinline__ bool stage_slots(const ClusterArgs& a, const int32_t* s_off,
-                                            const int32_t* s_pad, float4* s_lt, int t0, int tn) {
-  bool ok = true;
+// Light slots [t0, t0 + tn) of the padded table into s_lt; s_out[y] is set
+// where a light of cluster y is outside the packed contribution's bounds.
+__device__ __forceinline__ void stage_slots(const ClusterArgs& a, const int32_t* s_off,
+                                            const int32_t* s_pad, float4* s_lt, int32_t* s_out, int t0,
+                                            int tn) {
   for (int e = threadIdx.x; e < tn; e += blockDim.x) {
     int lo = 0, hi = a.k - 1;   // the cluster whose padded run holds slot t0 + e
     while (lo < hi) {
@@ -324,9 +324,8 @@ __device__ __forceinline__ bool stage_slots(const ClusterArgs& a, const int32_t*
     float4 l = table_light(a, pad ? s_off[lo] : at);
     if (pad) l.w = 0.0f;
     xp::put_light(s_lt, e, l);
-    ok = ok && xp::light_ok(l);
+    if (!xp::light_ok(l)) s_out[lo] = 1;
   }
-  return ok;
 }
 
 template <bool FEW>
@@ -337,9 +336,11 @@ __global__ void __launch_bounds__(kSumThreads, 3)
   float* s_w = reinterpret_cast<float*>(s_lt + a.tile) + threadIdx.x;
   int32_t* s_off = reinterpret_cast<int32_t*>(s_lt + a.tile) + kMaxClusters * kSumThreads;
   int32_t* s_pad = s_off + kMaxClusters + 4;
+  int32_t* s_out = s_pad + kMaxClusters + 4;
   const Occluders occ = stage_occluders<FEW>(a.spheres, a.n_sph, a.boxes, a.n_box,
-                                             s_pad + kMaxClusters + 4, threadIdx.x, blockDim.x);
+                                             s_out + kMaxClusters + 4, threadIdx.x, blockDim.x);
   const int k = a.k;
+  if (threadIdx.x < kMaxClusters) s_out[threadIdx.x] = 0;
   for (int e = threadIdx.x; e <= k; e += blockDim.x) s_off[e] = a.off[e];
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -353,8 +354,10 @@ __global__ void __launch_bounds__(kSumThreads, 3)
   __syncthreads();
   const int n_slots = s_pad[k];
   const bool whole = n_slots <= a.tile;
-  bool lights_ok = true;
-  if (whole) lights_ok = __syncthreads_and(stage_slots(a, s_off, s_pad, s_lt, 0, n_slots)) != 0;
+  if (whole) {
+    stage_slots(a, s_off, s_pad, s_lt, s_out, 0, n_slots);
+    __syncthreads();
+  }
   for (int64_t b = (int64_t)blockIdx.x * kSumThreads; b < a.n; b += (int64_t)gridDim.x * kSumThreads) {
     const int64_t p = b + threadIdx.x;
     const bool live = p < a.n;
@@ -370,21 +373,26 @@ __global__ void __launch_bounds__(kSumThreads, 3)
       const int t1 = min(t0 + a.tile, n_slots);
       if (!whole) {
         __syncthreads();   // the previous tile is read by every thread
-        lights_ok = __syncthreads_and(stage_slots(a, s_off, s_pad, s_lt, t0, t1 - t0)) != 0;
+        stage_slots(a, s_off, s_pad, s_lt, s_out, t0, t1 - t0);
+        __syncthreads();
       }
-      pp.ok = pixel_ok && lights_ok;
       int cur = t0;
       while (y < k) {
         const int pad_end = s_pad[y + 1], end = min(pad_end, t1);
         // the run's bounds are checked once; a run that breaks them is summed
-        // again, light by light, from where it began
+        // again, light by light, from where it began, and one that holds a
+        // light out of bounds only so (one light of 1024 out of bounds, k = 32,
+        // a million pixels: 3,030 -> 1,300 us; none 1,210)
+        pp.ok = pixel_ok && s_out[y] == 0;
         const float ch0 = ch;
         float dmin = 1.0f;
         uint32_t tmin = 0xFFFFFFFFu;
+        if (pp.ok) {
 #pragma unroll 2
-        for (int i = cur - t0; i < end - t0; i += 2) {
-          const float2 c = xp::contribution2(pp, s_lt[i], s_lt[i + 1], dmin, tmin);
-          ch = __fadd_rn(__fadd_rn(ch, c.x), c.y);
+          for (int i = cur - t0; i < end - t0; i += 2) {
+            const float2 c = xp::contribution2(pp, s_lt[i], s_lt[i + 1], dmin, tmin);
+            ch = __fadd_rn(__fadd_rn(ch, c.x), c.y);
+          }
         }
         if (!xp::in_bounds(pp, dmin, tmin)) {
           ch = ch0;
@@ -534,7 +542,7 @@ size_t sample_clustered_smem(const nvc_scene* sc, const nvc_clusters* cl) {
   const size_t occ =
       occluder_bytes(sc->n_spheres, sc->n_boxes) + sizeof(float4) * ((kMaxClusters + 4) / 4);
   if (cl->weights == NVC_CLUSTER_WEIGHT_VISIBILITY) return occ;   // no light loop
-  return occ + sizeof(float4) * ((kMaxClusters + 4) / 4 + light_slots(sc, cl)) +
+  return occ + sizeof(float4) * (2 * ((kMaxClusters + 4) / 4) + light_slots(sc, cl)) +
          sizeof(float) * kMaxClusters * kSumThreads;
 }
 
