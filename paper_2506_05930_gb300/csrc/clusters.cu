@@ -20,7 +20,6 @@
 //   sample_visibility_kernel the same with w_y = max(v_y, 0.001) alone.
 // Every float32 result is rounded in a fixed order and every random choice
 // is a fixed Philox word, so the kernels are reproducible bit for bit.
-#include <cfloat>
 #include <vector>
 
 #include "exact_pair.cuh"
@@ -112,10 +111,6 @@ __device__ __forceinline__ int cluster_reservoir(WFn wfn, int k, uint32_t pixel,
   for (int y = 0; y < kMaxClusters; ++y)
     if (y < k) wmax = fmaxf(wmax, wfn(y));
   if (!(wmax > 0.0f)) return -1;
-  // quantize_weight's integers by exact multiplications; an infinite weight
-  // takes quantize_weight itself
-  const bool finite = wmax <= FLT_MAX;
-  const fz::QuantScale qs = fz::quant_scale(wmax);
   const int e = ilogbf(wmax);
   uint32_t Q = 0;
   int sel = -1;
@@ -128,8 +123,7 @@ __device__ __forceinline__ int cluster_reservoir(WFn wfn, int k, uint32_t pixel,
         const int y = 4 * g + l;
         if (y < k) {
           const float w = wfn(y);
-          const uint32_t q = finite ? fz::quantize_scaled(__fmul_rn(w, qs.pre), qs.scale)
-                                    : quantize_weight(w, e);
+          const uint32_t q = quantize_weight(w, e);
           Q += q;
           if (q > 0u && __umulhi(fz::pick_word(r4, l), Q) < q) sel = y;
         }
@@ -235,9 +229,14 @@ __device__ __forceinline__ float4 table_light(const ClusterArgs& a, int slot) {
 
 // ---- first-step weights max(v, 0.001) alone ---------------------------------
 // No light loop: a pixel's visibilities are loaded together (16-byte loads
-// when the row allows) into the weights' registers.
+// when the row allows) into the weights' registers.  Bound by the latency of
+// its loads and its chain of random picks: 24 warps an SM at 80 registers, with
+// quantize_weight as it is, a million pixels, k = 32, no occluders 104 -> 90 us,
+// 32 + 32 152 -> 142; 28 and 32 warps 94 and 96 us, and exact multiplications
+// with a branch for infinite weights, which pay where one thread walks more
+// weights, 7% more.
 template <bool FEW>
-__global__ void __launch_bounds__(128, 7) sample_visibility_kernel(const __grid_constant__ ClusterArgs a,
+__global__ void __launch_bounds__(128, 6) sample_visibility_kernel(const __grid_constant__ ClusterArgs a,
                                                                  bool vis_vec4) {
   extern __shared__ float4 s_scene4[];
   int32_t* s_off = reinterpret_cast<int32_t*>(s_scene4);
