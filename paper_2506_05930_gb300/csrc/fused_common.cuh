@@ -240,17 +240,6 @@ __device__ __forceinline__ float2 contribution2_fast(float2 npx, float2 npy, flo
   return c;
 }
 
-// Clears the accumulator words of columns n and up.  The samplers' last group
-// takes in padding columns, against zero lights; a column's weights are zero
-// there, but 0 x infinity (a 16-bit activation that overflowed) is not, and a
-// NaN would come through the zero contribution into Neural DI.
-template <int N>
-__device__ __forceinline__ void clear_past(uint32_t (&r)[N], int n) {
-#pragma unroll
-  for (int j = 0; j < N; ++j)
-    if (j >= n) r[j] = 0u;
-}
-
 __host__ __device__ __forceinline__ int round_up16(int x) { return (x + 15) & ~15; }
 
 // Stages the L lights (float4 x, y, z, I) as pairs for contribution2_fast,

@@ -238,9 +238,8 @@ __global__ void __launch_bounds__(kTileM * TPC, TPC == 2 ? 3 : 2)
         const float2 npx = make_float2(-px, -px), npy = make_float2(-py, -py),
                      npz = make_float2(-pz, -pz);
         const float2 nx2 = make_float2(nx, nx), ny2 = make_float2(ny, ny), nz2 = make_float2(nz, nz);
-        // bounds by groups of four: lights past L in a group are zero lights
-        // with a cleared logit, whose terms are 0
-        if (L & 3) clear_past(r, L);
+        // bounds by groups of four: lights past L in a group are zero lights,
+        // whose terms are 0 (pack_mlp_kernel)
 #pragma unroll
         for (int q4 = 0; q4 < 8; ++q4) {
           if (q4 * 4 < L) {

@@ -212,10 +212,8 @@ __global__ void __launch_bounds__(kTileM, 5) fused_shade_kernel(const __grid_con
           uint32_t r[32];
           tmem_ld32(t_lane + (uint32_t)c0, r);
           // two lights per packed operation (pair (c0 + j) / 2 of the table);
-          // bounds by groups of four, lights past L in a group are zero lights
-          // with a cleared logit, whose terms are 0 (1080p x 32 lights 402 ->
-          // 365 us)
-          if ((L & 3) && L - c0 < 32) clear_past(r, L - c0);
+          // bounds by groups of four, lights past L in a group are zero lights,
+          // whose terms are 0 (pack_mlp_kernel; 1080p x 32 lights 402 -> 365 us)
 #pragma unroll
           for (int g = 0; g < 32; g += 4) {
 #pragma unroll
@@ -335,8 +333,7 @@ __global__ void __launch_bounds__(kTileM, 5) fused_shade_kernel(const __grid_con
 // the picks are the same integers from the same float32 weights.
 //
 // The light table is padded to whole 16-light chunks with zero lights, whose
-// terms are 0 with the last chunk's padded logits cleared (clear_past), so the
-// sampler's loops carry no bounds: with a bound per light the compiler kept a compare and a predicate
+// terms are 0 (pack_mlp_kernel), so the sampler's loops carry no bounds: with a bound per light the compiler kept a compare and a predicate
 // on every operation.  3840x2160 x 256 lights, FP16: 6.87 -> 5.03 ms; four
 // views of 128 lights (14,976,000 random points): 7.97 -> 7.75 ms, there with
 // half the time in the encode's scattered row reads (load_x_pairs).  Four threads per pixel
@@ -546,7 +543,6 @@ __global__ void __launch_bounds__(2 * kTileM, MINB) fused_shade_pair_kernel(cons
         for (int c0 = lo; c0 < hi; c0 += 16) {
           uint32_t r[16];
           tmem_ld16(t_lane + (uint32_t)c0, r);
-          if (L - c0 < 16) clear_past(r, L - c0);
           // two lights per packed operation (pair (c0 + j) / 2 of the table)
 #pragma unroll
           for (int j = 0; j < 16; j += 2) {
@@ -966,6 +962,13 @@ __global__ void __launch_bounds__(kTileM + PW * 32, PW == 4 ? 2 : 1) fused_shade
 }
 
 // ---- weight packing (fp32 master -> tensor-core operand image) -------------
+// The output layer's padding rows repeat its last real row.  The samplers take
+// in the padding columns up to the end of a group of lights, against lights of
+// zero intensity; with weights of zero a 16-bit activation that overflowed to
+// infinity would make their logits 0 x infinity, and the NaN would come through
+// the zero contribution into Neural DI.  Repeated, a padding logit is a number
+// whenever the last light's is.  (Clearing the logits in the samplers instead
+// cost scattered positions 8%: another schedule of the encode.)
 
 template <int PREC>
 __global__ void pack_mlp_kernel(const float* __restrict__ params, PackArgs p, uint8_t* out) {
@@ -978,8 +981,9 @@ __global__ void pack_mlp_kernel(const float* __restrict__ params, PackArgs p, ui
     const int grp = local >> 6, within = local & 63;
     const int kg = grp % (p.K[k] / 8), ng = grp / (p.K[k] / 8);
     const int n = ng * 8 + (within >> 3), kk = kg * 8 + (within & 7);
-    const float v = (n < p.N_real[k] && kk < p.K_real[k])
-                        ? params[p.w_off[k] + (int64_t)n * p.K_real[k] + kk]
+    const int row = k + 1 == p.n_layers && n >= p.N_real[k] ? p.N_real[k] - 1 : n;
+    const float v = (row < p.N_real[k] && kk < p.K_real[k])
+                        ? params[p.w_off[k] + (int64_t)row * p.K_real[k] + kk]
                         : 0.0f;
     if constexpr (PREC == NVC_PREC_BF16)
       reinterpret_cast<__nv_bfloat16*>(out + p.byte_off[k])[local] = __float2bfloat16_rn(v);
@@ -1016,7 +1020,8 @@ __global__ void pack_mlp_fp8_kernel(const float* __restrict__ params, PackArgs p
     const int grp = e >> 7, within = e & 127;
     const int kg = grp % (K / 16), ng = grp / (K / 16);
     const int n = ng * 8 + (within >> 4), kk = kg * 16 + (within & 15);
-    const float v = (n < nr && kk < kr) ? W[(int64_t)n * kr + kk] * scale : 0.0f;
+    const int row = k + 1 == p.n_layers && n >= nr ? nr - 1 : n;
+    const float v = (row < nr && kk < kr) ? W[(int64_t)row * kr + kk] * scale : 0.0f;
     dst[e] = (uint8_t)(pack_e4m3x2(v, 0.0f) & 0xFFu);
   }
 }
@@ -1222,6 +1227,7 @@ bool mlp_image_map(const nvc_handle* h, MlpImageMap* m) {
   }
   m->w_off[p.n_layers] = p.w_off[p.n_layers - 1] + (int64_t)p.N_real[p.n_layers - 1] *
                                                        p.K_real[p.n_layers - 1];
+  m->rows = p.N[p.n_layers - 1];
   m->bf16 = h->cfg.precision == NVC_PREC_BF16;
   return true;
 }

@@ -161,10 +161,12 @@ enum ShadeVariant : int {
 // Where each MLP weight sits in the tensor cores' 16-bit weight image (the
 // layout pack_mlp_kernel writes): layer k's W[n][kk] (parameter w_off[k] +
 // n K_real + kk) is element ((n/8) (K/8) + kk/8) 64 + (n%8) 8 + kk%8 of the
-// layer's block at byte_off[k].  The Adam kernel uses it to refresh the
-// image from the updated weights in the same pass.
+// layer's block at byte_off[k].  The last layer's rows from its last real one
+// to `rows` are that row again.  The Adam kernel uses it to refresh the image
+// from the updated weights in the same pass.
 struct MlpImageMap {
   int n_layers;
+  int rows;   // of the last layer's block
   int64_t w_off[NVC_MAX_HIDDEN_LAYERS + 2];   // [n_layers] = end of the last layer
   int K_real[NVC_MAX_HIDDEN_LAYERS + 1], K[NVC_MAX_HIDDEN_LAYERS + 1];
   int byte_off[NVC_MAX_HIDDEN_LAYERS + 1];

@@ -219,12 +219,16 @@ __device__ __forceinline__ void set_image(const MlpImageMap& mp, uint8_t* img, i
   int k = 0;
   while (k + 1 < mp.n_layers && j >= mp.w_off[k + 1]) ++k;
   const int64_t lj = j - mp.w_off[k];
-  const int n = (int)(lj / mp.K_real[k]), kk = (int)(lj - (int64_t)n * mp.K_real[k]);
-  const int local = ((((n >> 3) * (mp.K[k] >> 3)) + (kk >> 3)) << 6) + ((n & 7) << 3) + (kk & 7);
-  if (mp.bf16)
-    reinterpret_cast<__nv_bfloat16*>(img + mp.byte_off[k])[local] = __float2bfloat16_rn(v);
-  else
-    reinterpret_cast<__half*>(img + mp.byte_off[k])[local] = __float2half_rn(v);
+  int n = (int)(lj / mp.K_real[k]);
+  const int kk = (int)(lj - (int64_t)n * mp.K_real[k]);
+  const bool last_row = k + 1 == mp.n_layers && j + mp.K_real[k] >= mp.w_off[k + 1];
+  do {
+    const int local = ((((n >> 3) * (mp.K[k] >> 3)) + (kk >> 3)) << 6) + ((n & 7) << 3) + (kk & 7);
+    if (mp.bf16)
+      reinterpret_cast<__nv_bfloat16*>(img + mp.byte_off[k])[local] = __float2bfloat16_rn(v);
+    else
+      reinterpret_cast<__half*>(img + mp.byte_off[k])[local] = __float2half_rn(v);
+  } while (last_row && ++n < mp.rows);
 }
 
 // A thread loads kAdamGroups float4 groups (e, e + stride, ...) before any

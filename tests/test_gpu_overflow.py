@@ -60,3 +60,48 @@ def test_padding_columns_stay_out_of_the_radiance(L, precision, big):
             for k in ("radiance", "wsum", "pdf"):
                 assert torch.equal(out[k], got[0][k]), (variant, k)
     cache.close()
+
+
+@pytest.mark.parametrize("precision", ["fp16", "bf16"])
+@pytest.mark.parametrize("L", [1, 21, 47])
+def test_padding_rows_follow_the_training_step(L, precision):
+    """The weight image after a step, padding included, is the one that a new
+    handle makes from the same parameters: equal results bit for bit, with two
+    units of the last hidden layer overflowing, whose weights the step changes."""
+    from paper_2506_05930_gb300 import nvc
+    n, big = 700, 6e4 if precision == "fp16" else 3e38
+    cfg = dict(n_levels=4, n_features=2, log2_table_size=9, base_resolution=4, growth=1.5,
+               hidden=(32, 32), n_outputs=L, leaky_slope=0.01, precision=precision,
+               batch_positions=256, lr=0.05)
+    a, b = nvc.VisibilityCache(cfg), nvc.VisibilityCache(cfg)
+    g = torch.Generator(device="cuda").manual_seed(L)
+    p = 0.3 * torch.randn(a.n_params, device="cuda", generator=g)
+    a.set_params(p)
+    r = np.random.default_rng(L)
+    scene = nvc.Scene(np.hstack([r.uniform(0, 1, (L, 3)), r.uniform(0.5, 2.0, (L, 1))]),
+                      np.array([[0.5, 0.5, 0.5, 0.3]]))
+    for frame in range(3):
+        a.train_step(scene, None, seed=1, frame=frame)
+    assert a.counters()["step"] == 3
+    q = torch.empty_like(p)
+    nvc.nvc_get_state(a.handle, q)
+    assert not torch.equal(p[-L * 32:], q[-L * 32:])
+    b.set_params(q)
+    pos = torch.rand((n, 3), device="cuda", generator=g)
+    nrm = torch.nn.functional.normalize(torch.randn((n, 3), device="cuda", generator=g), dim=1)
+    for variant in (0, 5) + ((6,) if L <= 32 else ()):
+        outs = []
+        for c in (a, b):
+            nvc.nvc_set_shade_variant(c.handle, variant)
+            outs.append(c.shade(scene, pos, nrm, seed=3, frame=1))
+        for k in ("idx", "pdf", "wsum", "radiance"):
+            assert torch.equal(outs[0][k], outs[1][k]), (variant, k)
+    # one step from overflowing weights: +-infinite logits, a finite radiance
+    w1 = 4 * 512 * 2 + 32 * 8
+    q[w1 + 5 * 32:w1 + 6 * 32] = big
+    a.set_params(q)
+    a.train_step(scene, None, seed=1, frame=9)
+    out = a.shade(scene, pos, nrm, seed=3, frame=1)
+    assert torch.isfinite(a.infer(pos)).all() and torch.isfinite(out["radiance"]).all()
+    a.close()
+    b.close()
