@@ -241,6 +241,7 @@ __device__ __forceinline__ float2 contribution2_fast(float2 npx, float2 npy, flo
 }
 
 __host__ __device__ __forceinline__ int round_up16(int x) { return (x + 15) & ~15; }
+__host__ __device__ __forceinline__ int round_up4(int x) { return (x + 3) & ~3; }
 
 // Stages the L lights (float4 x, y, z, I) as pairs for contribution2_fast,
 // I scaled by 1/pi; slots from L to Lp (an even count) are zero lights.

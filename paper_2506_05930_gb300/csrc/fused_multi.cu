@@ -83,7 +83,7 @@ __global__ void __launch_bounds__(kTileM * TPC, TPC == 2 ? 3 : 2)
 
   for (int e = t; e < a.wimg_bytes / 16; e += kThreads)
     reinterpret_cast<uint4*>(s_w)[e] = a.wimg[e];
-  if (a.lights) stage_light_pairs(s_l, a.lights, a.L, t, kThreads, round_up16(a.L));
+  if (a.lights) stage_light_pairs(s_l, a.lights, a.L, t, kThreads, round_up4(a.L));
   if (t == 0) {
     for (int gg = 0; gg < TPC; ++gg) mbar_init(smem_u32(s_bar + gg), 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -355,7 +355,7 @@ size_t multi_smem(const nvc_handle* h, const PackArgs& p, int tpc, FusedArgs* a 
   stride = (stride + 127) & ~(size_t)127;
   off += (size_t)tpc * stride;
   const size_t l_off = off;
-  off += 16 * (size_t)round_up16(h->L > 0 ? h->L : 1);
+  off += 16 * (size_t)round_up4(h->L > 0 ? h->L : 1);
   off = (off + 7) & ~(size_t)7;
   const size_t bar_off = off;
   off += 8 * (size_t)tpc + 8 + 4 * (size_t)tpc;
