@@ -1300,35 +1300,54 @@ bool fused_supported(const nvc_handle* h, std::string* why) {
   return true;
 }
 
-// The layout of a launch whose handle has chosen none, by light count and
-// 128-pixel tiles.  All give the same picks; variants 0 and 6 also give the
-// same sums, which variant 5 adds by halves (see ShadeVariant).  So that a
+// The layout of a launch whose handle has chosen none, by light count, 128-pixel
+// tiles and table size.  All give the same picks; variants 0 and 6 also give
+// the same sums, which variant 5 adds by halves (see ShadeVariant).  So that a
 // pixel's outputs do not depend on how many others share its launch, the tile
 // count only chooses between layouts with the same sums: 0 and 6, and 5 among
 // them where one half holds every light (up to 16) or nothing is summed
-// (exported visibilities).  Measured in us, 16 levels x 2 features, MLP
-// 32-64-64-64-L, variants 0 / 5 / 6, shading of a heightfield:
-//   32 lights   1,000 px 18.7 / 15.3 / 20.8      9,728 px 18.6 / 15.2 / 20.6
-//              20,000 px 23.4 / 18.5 / 20.6     56,320 px 29.4 / 22.6 / 26.3
-//             129,600 px 43.6 / 36.9 / 37.3    578,731 px  122 /  128 /  111
-//   17 lights   9,728 px 18.6 / 15.0 / 20.9     20,000 px 22.5 / 18.5 / 20.6
-//   21 lights, float32 table                   578,731 px  113 /  130 /  107
-//   40 lights   4,096 px 21.1 / 17.1            76,800 px 37.7 / 33.6
-//                                              578,731 px  139 /  144
-//   96 lights                                  578,731 px  200 /  187
-// Few tiles are a chain of latencies, which two threads a pixel shorten;
-// many are bound by issue, where two tile streams per CTA keep most warps in
-// flight, from about one tile per SM on.  Above 32 lights variant 6 does not
-// run: two threads a pixel win from 64 lights, and for exported visibilities
-// (40 lights, 578,731 px: 133 against 123).  E4M3 operands run 0 and 5; 0 is
-// the faster from 1,000 px on.
+// (exported visibilities).
+//
+// What a launch waits for decides: its chain of latencies when the tiles are
+// few, which two threads a pixel shorten (3 tiles an SM and less); scattered
+// rows of a large table, which more warps in flight hide; else issue slots, of
+// which one thread a pixel wastes fewest.  Above 64 lights the sampler's loops
+// favour variant 5 either way, from 33 variant 6 does not run, exactly 32
+// lights have an instantiation of 6 without bounds, and four lights or fewer
+// fill neither 5 nor 6.  Times over variant 0's, 5 / 6 (MLP 64-64-64, half-
+// precision table; "large" 16 levels x 2^19 rows, "small" 16 x 2^17):
+//                       heightfield, 100,000 px     500,000 px    random points
+//   shading   4 large         1.14 / 1.10          1.32 / 1.09     0.99 / 1.12
+//             8 large         0.84 / 0.84          1.08 / 0.93     0.52 / 0.58
+//             8 small         1.06 / 0.98          1.27 / 1.12     0.52 / 0.57
+//            21 large         0.92 / 0.92          1.06 / 1.03     0.54 / 0.59
+//            21 small         1.11 / 1.00          1.22 / 1.11     0.56 / 0.58
+//            32 large         0.88 / 0.86          0.98 / 0.93     0.54 / 0.51
+//            32 small         1.06 / 0.95          1.13 / 1.01     0.56 / 0.52
+//           100 small         1.08 / -             1.07 / -        0.62 / -
+//   infer     8 large         0.74 / 0.83          0.90 / 0.91     0.51 / 0.59
+//             8 small         0.99 / 1.06          1.12 / 1.15     0.50 / 0.58
+//            21 large         0.78 / 0.86          0.87 / 0.88     0.53 / 0.61
+//            21 small         0.93 / 1.01          1.00 / 1.02     0.53 / 0.61
+//            32 small         1.00 / 0.93          1.08 / 0.97     0.52 / 0.48
+//            40 large         0.77 / -             0.90 / -        0.53 / -
+//            40 small         1.03 / -             1.08 / -        0.52 / -
+//           100 small         0.94 / -             0.93 / -        0.65 / -
+// E4M3 operands run 0 and 5; 0 is the faster from 1,000 px on.
 int default_variant(const nvc_handle* h, const PackArgs& p, const FusedArgs& a) {
   if (h->cfg.precision == NVC_PREC_FP8) return kShadeMono;
+  const int L = h->L;
   const bool infer = a.v[0].vis_out != nullptr;
-  const bool pair_fits = pair_smem(h, p) <= 225 * 1024;
-  if (h->L > 32) return (h->L > 64 || infer) && pair_fits ? kShadePair : kShadeMono;
-  if ((h->L <= 16 || infer) && a.n_tiles <= 3 * h->num_sms && pair_fits) return kShadePair;
-  return a.n_tiles > h->num_sms && multi_fits(h, p, 2) ? kShadeMulti2 : kShadeMono;
+  const bool few = a.n_tiles <= 3 * h->num_sms;
+  const bool large = ((int64_t)a.ep.n_levels << a.ep.log2_table) > (1 << 22);   // rows
+  const bool pair = L > 64                    ? true
+                    : infer && L > 32         ? few || large
+                    : infer && L < 32         ? few || L > 15 || (large && L > 4)
+                                              : few && (infer || L <= 16);
+  if (pair) return pair_smem(h, p) <= 225 * 1024 ? kShadePair : kShadeMono;
+  const bool multi = L == 32 || (!infer && large && L > 4 && L < 32);
+  return multi && a.n_tiles > (large ? 1 : 3) * h->num_sms && multi_fits(h, p, 2) ? kShadeMulti2
+                                                                                  : kShadeMono;
 }
 
 cudaError_t launch_shade_fused_views(const nvc_handle* h, const nvc_scene* sc,
