@@ -473,10 +473,9 @@ nvc_status nvc_cluster_targets(const nvc_scene* scene, const nvc_clusters* clust
  * vis: device [n][k], the cache's cluster visibilities (nvc_infer).
  * light (device [n], -1 when nothing contributes), weight (W) and estimate
  * (V(x) c(x) W with one shadow ray, 0 when blocked) may each be NULL.
- * Pixel ids are pixel_offset + p.  The scene's lights are staged in shared
- * memory when they fit beside the occluders (about 14,000 lights), else
- * read from global memory; step 1 costs one contribution per light and
- * pixel.  Asynchronous. */
+ * Pixel ids are pixel_offset + p.  For SUM the scene's lights are staged in
+ * shared memory, in tiles of 1,024; step 1 costs one contribution per light
+ * and pixel.  Asynchronous. */
 nvc_status nvc_sample_clustered(const nvc_scene* scene, const nvc_clusters* clusters,
                                 const float* vis, const float* pos, const float* nrm, int64_t n,
                                 int64_t pixel_offset, uint64_t seed, uint32_t frame,
