@@ -56,13 +56,14 @@ __global__ void __launch_bounds__(256) shade_estimate_kernel(
 
 // One light at a time for the whole warp (warp_segments_blocked), its
 // contribution two lights per packed operation (exact_pair.cuh).  A warp whose
-// pixels are not neighbours -- a light's vote keeps more than an eighth of the
-// occluders -- takes segment_blocked from there on, so the votes cost it one
-// ballot a 32 occluders (a million pixels x 8 lights, 32 + 32: 128 us, with the
-// limit at a half and the kept ones tested first 147; random positions 395 and
-// 457; 4,096 pixels x 32 lights, 500 + 500: 340 and 1,008).
-// 1920x1080 x 32 lights, 32 spheres + 32 boxes: 2.80 -> 0.757 ms; bound by
-// instruction issue (9,900 a warp and 32 lights; 75% of the slots).
+// pixels are not neighbours -- a light's vote keeps more than a quarter of the
+// occluders -- takes segment_blocked from there on, so the votes cost it that
+// many tests.
+// 1920x1080 x 32 lights, 32 spheres + 32 boxes: 2.80 -> 0.756 ms; bound by
+// instruction issue (9,900 a warp and 32 lights; 75% of the slots).  With the
+// limit at an eighth 0.773, at a half, left only after every kept occluder's
+// test, 0.760, and 4,096 pixels x 32 lights, 500 + 500, 1,009 us where a
+// quarter takes 515 (every occluder tested: 654).
 // kSmemLights: the lights (with I / pi) are staged after the occluders as
 // pairs, in groups of four with zero lights past the last; otherwise they are
 // read through the read-only cache and scaled here (the same rounding), for
@@ -87,7 +88,7 @@ __global__ void __launch_bounds__(256, 3) exact_di_kernel(
     }
   }
   lights_ok = __syncthreads_and(lights_ok) != 0;
-  const int limit = (2 * occ.n_pairs + occ.n_box) / 8 + 2;
+  const int limit = (2 * occ.n_pairs + occ.n_box) / 4 + 2;
   // whole warps walk the pixels: a lane past the end repeats the warp's first
   // pixel and writes nothing
   for (int64_t p0 = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); p0 < n;

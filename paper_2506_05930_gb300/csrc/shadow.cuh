@@ -456,8 +456,8 @@ __device__ __forceinline__ bool hull_meets_box(const WarpHull& w, const HullRay&
 }
 
 // segment_blocked for a whole warp looking at one light: *blocked is the
-// answer of the lanes with `want`.  Gives up, with false in every lane, when
-// more than `limit` occluders would have to be tested exactly.
+// answer of the lanes with `want`.  Gives up, with false in every lane, after
+// `limit` exact tests.
 __device__ __forceinline__ bool warp_segments_blocked(const WarpHull& w, bool want, float px, float py,
                                                       float pz, float lx, float ly, float lz,
                                                       const Occluders& occ, int limit, bool* blocked) {
@@ -468,18 +468,16 @@ __device__ __forceinline__ bool warp_segments_blocked(const WarpHull& w, bool wa
   *blocked = want;   // until the last occluder is past with lanes still open
   for (int b = 0; b < 2 * occ.n_pairs; b += 32) {
     const bool near = b + lane < 2 * occ.n_pairs && hull_meets_sphere(w, r, occ, b + lane);
-    unsigned m = __ballot_sync(0xffffffffu, near);
-    if ((limit -= __popc(m)) < 0) return false;
-    for (; m; m &= m - 1) {
+    for (unsigned m = __ballot_sync(0xffffffffu, near); m; m &= m - 1) {
+      if (--limit < 0) return false;
       open = open && !sphere_blocks(g, occ, b + __ffs(m) - 1);
       if (!__any_sync(0xffffffffu, open)) return true;
     }
   }
   for (int b = 0; b < occ.n_box; b += 32) {
     const bool near = b + lane < occ.n_box && hull_meets_box(w, r, occ, b + lane);
-    unsigned m = __ballot_sync(0xffffffffu, near);
-    if ((limit -= __popc(m)) < 0) return false;
-    for (; m; m &= m - 1) {
+    for (unsigned m = __ballot_sync(0xffffffffu, near); m; m &= m - 1) {
+      if (--limit < 0) return false;
       open = open && !box_blocks(g, occ, b + __ffs(m) - 1);
       if (!__any_sync(0xffffffffu, open)) return true;
     }
