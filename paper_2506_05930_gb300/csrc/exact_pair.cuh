@@ -10,7 +10,8 @@
 // lights at once:
 //   s = g + (x - g g) r / 2,          g = x r, r ~ 1 / sqrt(x);
 //   y = y0 + (1 - b y0) y0, y0 ~ 1/b; q = a y;  q + (a - b q) y.
-// Checked on the device against the library's: s for every float of
+// Checked on the device against the library's (test_gpu_exact_arithmetic.py
+// repeats it, the quotients in part): s for every float of
 // [2^-20, 2^64), the quotient for all 2^46 pairs of mantissas; both scale
 // with powers of two while nothing leaves the normal range, which the bounds
 // below guarantee.  A group of lights outside them takes contribution().
